@@ -273,6 +273,29 @@ struct copy_scope {
 
 int sm_count();
 
+// Programmatic dependent launch: a kernel started with launch_pdl may be
+// set up while the kernel before it on the stream still runs; it calls
+// pdl_wait before it touches memory, which holds it until that kernel has
+// finished and its writes are visible.  pdl_trigger lets the next one be set
+// up (it only starts once every CTA of this kernel is running or done).
+// Plain launches on the same stream order as ever.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // build pieces (tc_build.cu)
 tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np, int64_t n,
                       uint32_t flags, cudaStream_t s);

@@ -1,0 +1,69 @@
+"""Kernels at the sizes where their tiles, units and rules end: each case
+against the oracle, bit for bit."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+import graphgen as gg
+import oracle
+import paper_2105_00110_gb300 as tcg
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    tcg.build()
+    torch.cuda.init()
+
+
+def csr_rows(rows):
+    row_ptr = np.zeros(len(rows) + 1, np.int64)
+    np.cumsum([len(r) for r in rows], out=row_ptr[1:])
+    return row_ptr, np.array([c for r in rows for c in r], np.int32)
+
+
+def noalloc(row_ptr, col, n):
+    out = [torch.full((n,), 7, dtype=torch.int64, device="cuda").view(torch.uint64) for _ in range(2)]
+    tc = torch.full((n,), 7.0, dtype=torch.float64, device="cuda")
+    tcg.tc_csr_centrality_noalloc(torch.from_numpy(row_ptr).cuda(), torch.from_numpy(col).cuda(), n, *out, tc)
+    return [x.cpu().numpy() for x in (*out, tc)]
+
+
+def star(leaves):
+    """A hub, its leaves and one triangle on it."""
+    a = np.concatenate([np.zeros(leaves, np.int32), [1]]).astype(np.int32)
+    b = np.concatenate([np.arange(1, leaves + 1), [2]]).astype(np.int32)
+    return a, b, leaves + 1
+
+
+@pytest.mark.parametrize("graph", [
+    (np.zeros(0, np.int32), np.zeros(0, np.int32), 1),
+    (np.array([0], np.int32), np.array([1], np.int32), 2),
+    gg.complete_graph(17), gg.complete_graph(33),
+    star(255), star(256), star(1000),            # rows around the gather's whole-CTA rows
+    gg.gnp(65, 0.2, 5), gg.gnp(130, 0.5, 6),     # more than one bitmap word a row, ragged units
+    gg.rmat(13, 16, seed=7), gg.rmat(15, 14, seed=8),   # units of 16 and of 32 entries
+], ids=lambda g: "n%d-p%d" % (g[2], len(g[0])))
+def test_allocation_free_units(graph):
+    s, d, n = graph
+    ref = oracle.run(s, d, n)
+    tri, numer, tc = noalloc(ref["ptr"].astype(np.int64), ref["adj"].astype(np.int32), n)
+    assert np.array_equal(tri, ref["tri"]) and np.array_equal(numer, ref["numer"])
+    assert np.array_equal(tc, ref["tc"], equal_nan=True)
+
+
+@pytest.mark.parametrize("rows", [
+    [[0, 1], [0], []],                           # a loop
+    [[1, 1], [0, 0]],                            # repeated entries
+    [[1], [0], [3], []],                         # one-sided
+    [[1, 2, 3, 4, 5], [0], [0], [], [], []],     # three of five one-sided
+], ids=["loop", "repeat", "one-sided", "hub-one-sided"])
+def test_allocation_free_rejects(rows):
+    row_ptr, col = csr_rows(rows)
+    if len(col) & 1:
+        col, row_ptr = np.append(col, 0).astype(np.int32), np.append(row_ptr[:-1], len(col) + 1)
+    tri, numer, tc = noalloc(row_ptr, col, len(rows))
+    assert (tri.view(np.int64) == -1).all() and (numer.view(np.int64) == -1).all() and np.isnan(tc).all()
