@@ -75,20 +75,34 @@ __global__ void k_edges_degrees(const uint64_t* __restrict__ ukeys, int64_t m, i
 }
 
 __global__ void k_rank_keys(const int32_t* __restrict__ deg, int64_t n, int bits,
-                            uint64_t* __restrict__ keys) {
+                            uint64_t* __restrict__ keys, int64_t* __restrict__ band) {
+    if (blockIdx.x == 0 && threadIdx.x < 2) band[threadIdx.x] = n;   // lowered by k_rank_apply
     GRID_STRIDE(v, n) keys[v] = ((uint64_t)deg[v] << bits) | (uint64_t)v;
 }
 
+// Degree bands of the rows: degrees ascend with rank, and rows of degree up
+// to 32, up to TC_BAND_CTA and above take one thread, one warp and one CTA
+// each in the gather and the per-row work.  band[k] is the first rank above
+// limit k (n if none): the rank whose degree is the first to pass it.
+#ifndef TC_BAND_CTA
+#define TC_BAND_CTA 4096
+#endif
 __global__ void k_rank_apply(const uint64_t* __restrict__ sorted, int64_t n, int bits,
                              int32_t* __restrict__ perm, int32_t* __restrict__ rank,
-                             int64_t* __restrict__ degr) {
+                             int64_t* __restrict__ degr, int64_t* __restrict__ band) {
     const uint64_t mask = (1ull << bits) - 1;
     GRID_STRIDE(r, n) {
         uint64_t k = sorted[r];
         int32_t v = (int32_t)(k & mask);
         perm[r] = v;
         rank[v] = (int32_t)r;
-        degr[r] = (int64_t)(k >> bits);
+        const int64_t d = (int64_t)(k >> bits);
+        degr[r] = d;
+        if (d > 32) {
+            const int64_t before = r ? (int64_t)(sorted[r - 1] >> bits) : 0;
+            if (before <= 32) band[0] = r;
+            if (d > TC_BAND_CTA && before <= TC_BAND_CTA) band[1] = r;
+        }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) degr[n] = 0;
 }
@@ -112,8 +126,9 @@ __global__ void k_edge_rank_keys(const int32_t* __restrict__ eu, const int32_t* 
 template <class C>
 __global__ void k_hstart(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ dh,
                          const int64_t* __restrict__ hptr, int64_t n, int64_t* __restrict__ hstart,
-                         C* __restrict__ hnext, C* __restrict__ tnext) {
+                         C* __restrict__ hnext, C* __restrict__ tnext, int64_t* __restrict__ work) {
     GRID_STRIDE(r, n) {
+        work[r] = 0;   // k_row_work adds to it
         hstart[r] = row_ptr[r + 1] - dh[r];
         hnext[r] = (C)row_ptr[r];
         tnext[r] = (C)hptr[r];
@@ -578,24 +593,6 @@ k_runs_big(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hsta
     }
 }
 
-// First ranks whose degree exceeds 32 and TC_BAND_CTA (degrees ascend with
-// rank): the gather and the per-row work take one thread, one warp and one
-// CTA per row in the three bands.
-#ifndef TC_BAND_CTA
-#define TC_BAND_CTA 4096
-#endif
-__global__ void k_bands(const int64_t* __restrict__ row_ptr, int64_t n, int64_t* __restrict__ band) {
-    const int64_t lim[2] = {32, TC_BAND_CTA};
-    for (int k = 0; k < 2; ++k) {
-        int64_t lo = 0, hi = n;
-        while (lo < hi) {
-            const int64_t mid = lo + ((hi - lo) >> 1);
-            if (row_ptr[mid + 1] - row_ptr[mid] > lim[k]) hi = mid; else lo = mid + 1;
-        }
-        band[k] = lo;
-    }
-}
-
 // ------------------------------------------------------------ row work
 struct row_stats {
     unsigned long long sum_h2, wedges, sum_dh, max_h, max_d;
@@ -603,12 +600,16 @@ struct row_stats {
 
 // W(v) = Σ_{u ∈ N_L(v)} hrem(u, v), the number of ids the count step
 // streams for middle vertex v, plus shape statistics.  Rows ascend in
-// degree: rows below band[0] (degree <= 32) take one thread each, the rest
-// one warp each.
-// Rows of degree above 4096 get one CTA each in the per-row work (below).
-#ifndef TC_ROW_WORK_CTA
-#define TC_ROW_WORK_CTA 1
-#endif
+// degree: one launch takes the rows from band[0] on with a warp each, the
+// rest with a thread, and first the CSR positions of the rows from band[1]
+// on (hubs, up to hundreds of thousands of head entries) in segments of
+// kRowSegment, a warp each, added into work (zeroed beforehand): with a CTA a
+// row the largest hub alone took 0.55 ms on the 4096^2 grid.  It reads every
+// head record once.  The statistics are reduced per CTA before the five atomics: with
+// one set a warp, 10^5 atomics on five addresses took 33 + 18 us of the R-MAT
+// scale-12 pass and 0.13 ms at scales 16 and 20.
+constexpr int kRowWarps = kThreads / 32;
+constexpr int64_t kRowSegment = 2048;
 struct row_acc {
     unsigned long long h2 = 0, w = 0, dh = 0, maxh = 0, maxd = 0;
     __device__ __forceinline__ void add(unsigned long long hv, unsigned long long d, unsigned long long wr) {
@@ -618,94 +619,93 @@ struct row_acc {
         maxh = maxh > hv ? maxh : hv;
         maxd = maxd > d ? maxd : d;
     }
-    __device__ __forceinline__ void flush(row_stats* st) {
-        for (int o = 16; o; o >>= 1) {
-            h2 += __shfl_xor_sync(0xffffffffu, h2, o);
-            w += __shfl_xor_sync(0xffffffffu, w, o);
-            dh += __shfl_xor_sync(0xffffffffu, dh, o);
-            const unsigned long long a = __shfl_xor_sync(0xffffffffu, maxh, o);
-            const unsigned long long c = __shfl_xor_sync(0xffffffffu, maxd, o);
-            maxh = maxh > a ? maxh : a;
-            maxd = maxd > c ? maxd : c;
-        }
-        if ((threadIdx.x & 31) == 0) {
-            atomicAdd(&st->sum_h2, h2);
-            atomicAdd(&st->wedges, w);
-            atomicAdd(&st->sum_dh, dh);
-            atomicMax(&st->max_h, maxh);
-            atomicMax(&st->max_d, maxd);
-        }
+    __device__ __forceinline__ void join(const row_acc& o) {
+        h2 += o.h2;
+        w += o.w;
+        dh += o.dh;
+        maxh = maxh > o.maxh ? maxh : o.maxh;
+        maxd = maxd > o.maxd ? maxd : o.maxd;
     }
 };
 
-__global__ void k_row_work_thread(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart,
-                                  const tc_head* __restrict__ head, const int64_t* __restrict__ band,
-                                  int64_t* __restrict__ work, row_stats* __restrict__ st) {
-    const int64_t r1 = band[0];
-    row_acc acc;
-    // whole warps step together so that the final shuffles see every lane
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t warp_first = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) & ~31ll;
-    for (int64_t base = warp_first; base < r1; base += stride) {
-        const int64_t r = base + (threadIdx.x & 31);
-        if (r < r1) {
-            const int64_t b = row_ptr[r], h = hstart[r], e = row_ptr[r + 1];
-            unsigned long long w = 0;
-            for (int64_t p = b; p < h; ++p) w += (unsigned long long)head[p].hrem;
-            work[r] = (int64_t)w;
-            acc.add((unsigned long long)(e - h), (unsigned long long)(e - b), w);
-        }
-    }
-    acc.flush(st);
+__device__ __forceinline__ unsigned long long warp_sum64(unsigned long long w) {
+    for (int o = 16; o; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    return w;
 }
 
-__global__ void k_row_work_warp(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart,
-                                const tc_head* __restrict__ head, const int64_t* __restrict__ band, int64_t n,
-                                int64_t* __restrict__ work, row_stats* __restrict__ st) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+__global__ void __launch_bounds__(kThreads)
+k_row_work(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart, const tc_head* __restrict__ head,
+           const int64_t* __restrict__ band, int64_t n, int64_t* __restrict__ work, row_stats* __restrict__ st) {
+    __shared__ row_acc s_acc[kRowWarps];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const int64_t b0 = band[0], b1 = band[1];
+    const int64_t warps = (int64_t)gridDim.x * kRowWarps, w0 = (int64_t)blockIdx.x * kRowWarps + wp;
     row_acc acc;
-    const int64_t r1 = TC_ROW_WORK_CTA ? band[1] : n;   // rows above degree 4096: k_row_work_cta
-    for (int64_t r = band[0] + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5); r < r1; r += warps) {
+    const int64_t first = row_ptr[b1], last = row_ptr[n];
+    for (int64_t x0 = first + w0 * kRowSegment; x0 < last; x0 += warps * kRowSegment) {
+        const int64_t x1 = x0 + kRowSegment < last ? x0 + kRowSegment : last;
+        // row of position x0: the last one that starts at or before it
+        int64_t lo = b1, hi = n;
+        while (hi - lo > 1) {
+            const int64_t step = (hi - lo + 31) >> 5, x = lo + lane * step;
+            const unsigned m = __ballot_sync(0xffffffffu, x < hi && row_ptr[x] <= x0) | 1u;
+            lo += (31 - __clz(m)) * step;
+            hi = hi < lo + step ? hi : lo + step;
+        }
+        for (int64_t r = lo; r < n; ++r) {
+            const int64_t b = row_ptr[r], h = hstart[r], e = row_ptr[r + 1];
+            if (b >= x1) break;
+            const int64_t q1 = h < x1 ? h : x1;
+            unsigned long long w = 0;
+#pragma unroll 4
+            for (int64_t p = (b > x0 ? b : x0) + lane; p < q1; p += 32) w += (unsigned long long)head[p].hrem;
+            w = warp_sum64(w);
+            if (lane == 0) {
+                if (w) atomicAdd((unsigned long long*)&work[r], w);
+                acc.w += w;
+                if (b >= x0) acc.add((unsigned long long)(e - h), (unsigned long long)(e - b), 0);
+            }
+        }
+    }
+    for (int64_t r = b1 - 1 - w0; r >= b0; r -= warps) {
         const int64_t b = row_ptr[r], h = hstart[r], e = row_ptr[r + 1];
         unsigned long long w = 0;
+#pragma unroll 4
         for (int64_t p = b + lane; p < h; p += 32) w += (unsigned long long)head[p].hrem;
-        for (int o = 16; o; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+        w = warp_sum64(w);
         if (lane == 0) {
             work[r] = (int64_t)w;
             acc.add((unsigned long long)(e - h), (unsigned long long)(e - b), w);
         }
     }
-    acc.flush(st);
-}
-
-// Rows of degree above 4096 (ranks band[1] .. n - 1, the hubs, up to
-// hundreds of thousands of head entries each): one CTA per row, so that
-// the last hub rows do not each keep a single warp busy after the rest.
-__global__ void __launch_bounds__(512) k_row_work_cta(const int64_t* __restrict__ row_ptr,
-                                                      const int64_t* __restrict__ hstart,
-                                                      const tc_head* __restrict__ head,
-                                                      const int64_t* __restrict__ band, int64_t n,
-                                                      int64_t* __restrict__ work, row_stats* __restrict__ st) {
-    __shared__ unsigned long long part[16];
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    row_acc acc;
-    for (int64_t r = band[1] + blockIdx.x; r < n; r += gridDim.x) {
+    GRID_STRIDE(r, b0) {
         const int64_t b = row_ptr[r], h = hstart[r], e = row_ptr[r + 1];
         unsigned long long w = 0;
-        for (int64_t p = b + threadIdx.x; p < h; p += blockDim.x) w += (unsigned long long)head[p].hrem;
-        for (int o = 16; o; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-        if (lane == 0) part[wp] = w;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long s = 0;
-            for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += part[k];
-            work[r] = (int64_t)s;
-            acc.add((unsigned long long)(e - h), (unsigned long long)(e - b), s);
-        }
-        __syncthreads();
+        for (int64_t p = b; p < h; ++p) w += (unsigned long long)head[p].hrem;
+        work[r] = (int64_t)w;
+        acc.add((unsigned long long)(e - h), (unsigned long long)(e - b), w);
     }
-    acc.flush(st);
+    for (int o = 16; o; o >>= 1) {
+        row_acc x;
+        x.h2 = __shfl_xor_sync(0xffffffffu, acc.h2, o);
+        x.w = __shfl_xor_sync(0xffffffffu, acc.w, o);
+        x.dh = __shfl_xor_sync(0xffffffffu, acc.dh, o);
+        x.maxh = __shfl_xor_sync(0xffffffffu, acc.maxh, o);
+        x.maxd = __shfl_xor_sync(0xffffffffu, acc.maxd, o);
+        acc.join(x);
+    }
+    if (lane == 0) s_acc[wp] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < kRowWarps; ++k) acc.join(s_acc[k]);
+        if (acc.maxd) {   // some row with entries
+            atomicAdd(&st->sum_h2, acc.h2);
+            atomicAdd(&st->wedges, acc.w);
+            atomicAdd(&st->sum_dh, acc.dh);
+            atomicMax(&st->max_h, acc.maxh);
+            atomicMax(&st->max_d, acc.maxd);
+        }
+    }
 }
 
 int bits_for(int64_t n) {
@@ -757,7 +757,7 @@ tc_status build_runs(tc_graph* g, cudaStream_t s, int64_t m, int64_t n, int bits
                      C* hnext, C* tnext, int rows_blocks, int64_t core_t) {
     {
         launch_scope ls("build_hstart", s);
-        k_hstart<<<grid_for(n), kThreads, 0, s>>>(g->row_ptr, dh, hptr, n, g->hstart, hnext, tnext);
+        k_hstart<<<grid_for(n), kThreads, 0, s>>>(g->row_ptr, dh, hptr, n, g->hstart, hnext, tnext, g->work);
         TC_LAUNCH_CHECK();
     }
     {
@@ -902,6 +902,7 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
     TC_TRY(dalloc((void**)&g->hstart, (n + 1) * 8, s));
     TC_TRY(dalloc((void**)&g->head, (e2 + 1) * sizeof(tc_head), s));
     TC_TRY(dalloc((void**)&g->edge_tail, (m + 1) * 8, s));
+    TC_TRY(dalloc((void**)&g->work, (n + 1) * 8, s));
     TC_TRY(dalloc((void**)&g->tri, (n + 1) * 8, s));
     TC_TRY(dalloc((void**)&g->tri32, (n + 1) * 4, s));
     TC_TRY(dalloc((void**)&g->flag, flag_words(e2) * 4, s));
@@ -917,7 +918,8 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
         TC_LAUNCH_CHECK();
     }
     int32_t* rank = nullptr;
-    int64_t* degr = nullptr;
+    int64_t *degr = nullptr, *d_band = nullptr;
+    TC_TRY(sc.get(&d_band, 2));
     TC_TRY(sc.get(&rank, n + 1));
     TC_TRY(sc.get(&degr, n + 2));
     if (n > 0) {
@@ -926,7 +928,7 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
         TC_TRY(sc.get(&rb, n));
         {
             launch_scope ls("build_rank_keys", s);
-            k_rank_keys<<<grid_for(n), kThreads, 0, s>>>(deg, n, bits, ra);
+            k_rank_keys<<<grid_for(n), kThreads, 0, s>>>(deg, n, bits, ra, d_band);
             TC_LAUNCH_CHECK();
         }
         // the sort key is (degree << bits | label): it needs only as many
@@ -952,10 +954,11 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
             TC_TRY(sort_keys(sc, rbuf, n, bits + bits_for((int64_t)maxdeg + 1), s));
         }
         launch_scope ls("build_rank_apply", s);
-        k_rank_apply<<<grid_for(n), kThreads, 0, s>>>(rbuf.Current(), n, bits, g->perm, rank, degr);
+        k_rank_apply<<<grid_for(n), kThreads, 0, s>>>(rbuf.Current(), n, bits, g->perm, rank, degr, d_band);
         TC_LAUNCH_CHECK();
     } else {
         TC_CUDA(cudaMemsetAsync(degr, 0, 8, s));
+        TC_CUDA(cudaMemsetAsync(d_band, 0, 2 * 8, s));
     }
     {
         size_t bytes = 0;
@@ -1022,39 +1025,14 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
     }
 
     // ---- 6. per-row work, statistics and the count-step plan
-    TC_TRY(dalloc((void**)&g->work, (n + 1) * 8, s));
     row_stats* dst_stats = nullptr;
     TC_TRY(sc.get(&dst_stats, 1));
     TC_CUDA(cudaMemsetAsync(dst_stats, 0, sizeof(row_stats), s));
-    int64_t* d_band = nullptr;
-    TC_TRY(sc.get(&d_band, 2));
-    {
-        launch_scope ls("build_bands", s);
-        k_bands<<<1, 1, 0, s>>>(g->row_ptr, n, d_band);
-        TC_LAUNCH_CHECK();
-    }
     if (n > 0) {
-        const int cap = sm_count() * 16;
-        {
-            launch_scope ls("build_row_work_thread", s);
-            const int bt = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, (int64_t)cap);
-            k_row_work_thread<<<std::max(bt, 1), kThreads, 0, s>>>(g->row_ptr, g->hstart, g->head, d_band,
-                                                                   g->work, dst_stats);
-            TC_LAUNCH_CHECK();
-        }
-        {
-            launch_scope ls("build_row_work_warp", s);
-            const int bw = (int)std::min<int64_t>((n * 32 + kThreads - 1) / kThreads, (int64_t)cap);
-            k_row_work_warp<<<std::max(bw, 1), kThreads, 0, s>>>(g->row_ptr, g->hstart, g->head, d_band, n,
-                                                                 g->work, dst_stats);
-            TC_LAUNCH_CHECK();
-        }
-        if (TC_ROW_WORK_CTA) {
-            launch_scope ls("build_row_work_cta", s);
-            k_row_work_cta<<<sm_count() * 4, 512, 0, s>>>(g->row_ptr, g->hstart, g->head, d_band, n, g->work,
-                                                          dst_stats);
-            TC_LAUNCH_CHECK();
-        }
+        launch_scope ls("build_row_work", s);
+        const int blocks = (int)std::min<int64_t>((n + kRowWarps - 1) / kRowWarps, (int64_t)sm_count() * 8);
+        k_row_work<<<blocks, kThreads, 0, s>>>(g->row_ptr, g->hstart, g->head, d_band, n, g->work, dst_stats);
+        TC_LAUNCH_CHECK();
     }
     row_stats hst{};
     TC_CUDA(cudaMemcpyAsync(&hst, dst_stats, sizeof(row_stats), cudaMemcpyDeviceToHost, s));

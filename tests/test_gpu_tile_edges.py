@@ -67,3 +67,49 @@ def test_allocation_free_rejects(rows):
         col, row_ptr = np.append(col, 0).astype(np.int32), np.append(row_ptr[:-1], len(col) + 1)
     tri, numer, tc = noalloc(row_ptr, col, len(rows))
     assert (tri.view(np.int64) == -1).all() and (numer.view(np.int64) == -1).all() and np.isnan(tc).all()
+
+
+def check_full(src, dst, n):
+    """One full pass against the oracle, and the plan's wedge count against
+    the out-degrees of the degree order."""
+    res = tcg.triangle_centrality(torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), n)
+    ref = oracle.run(src, dst, n)
+    assert res["total"] == ref["total"]
+    for k in ("tri", "numer"):
+        assert np.array_equal(res[k].cpu().numpy(), ref[k][:n]), k
+    assert np.array_equal(res["tc"].cpu().numpy(), ref["tc"][:n], equal_nan=True)
+    rows = np.repeat(np.arange(n, dtype=np.int64), np.diff(ref["ptr"]))
+    keep = ref["adj"] > rows
+    u, v = rows[keep], ref["adj"][keep].astype(np.int64)
+    assert np.array_equal(res["edge_u"].cpu().numpy(), u) and np.array_equal(res["edge_v"].cpu().numpy(), v)
+    assert np.array_equal(res["flag"].cpu().numpy(), ref["flag"][keep])
+    deg = np.bincount(np.concatenate([u, v]), minlength=n)
+    rank = np.empty(n, np.int64)
+    rank[np.argsort(deg, kind="stable")] = np.arange(n)
+    dh = np.bincount(np.minimum(rank[u], rank[v]), minlength=n)
+    st = res["stats"]
+    assert st["wedges"] == float((dh * (dh - 1) // 2).sum()) and st["max_out_degree"] == dh.max(initial=0)
+    assert st["max_degree"] == deg.max(initial=0) and st["sum_out_degree_sq"] == float((dh * dh).sum())
+    assert sum(st["class_wedges"]) == st["wedges"]
+    return res
+
+
+def wheels(*rims):
+    """Hubs, each joined to every vertex of a cycle of its own; the hubs are
+    chained."""
+    src, dst, n = [], [], len(rims)
+    for h, r in enumerate(rims):
+        rim = np.arange(n, n + r)
+        src += [np.full(r, h), rim]
+        dst += [rim, np.roll(rim, 1)]
+        n += r
+    src.append(np.arange(1, len(rims)))
+    dst.append(np.arange(len(rims) - 1))
+    return np.concatenate(src).astype(np.int32), np.concatenate(dst).astype(np.int32), n
+
+
+# hub rows (degree above 4096) are walked in segments of 2048 positions
+@pytest.mark.parametrize("rims", [(4093,), (4097,), (4098, 6144), (20001, 4100, 33), (8192, 8191, 8190)],
+                         ids=lambda r: "-".join(map(str, r)))
+def test_hub_rows(rims):
+    check_full(*wheels(*rims))
