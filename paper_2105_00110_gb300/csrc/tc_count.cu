@@ -35,8 +35,6 @@
 // edge-count mode (EC), which adds per-entry triangle counts where the
 // normal mode sets flag bits, and an item offset/stride, which restricts a
 // launch to one shard's share of the items.
-#include <cub/cub.cuh>
-
 #include <algorithm>
 #include <mutex>
 #include <type_traits>
@@ -1042,92 +1040,159 @@ struct class_acc {
                                              // for the thread class: the largest |N_H(v)|)
 };
 
-// Class and chunk count of every middle vertex; rows visited in reverse
-// rank order so that the heaviest vertices come first in every class.
-__global__ void k_classify(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart,
-                           const int32_t* __restrict__ col, const int64_t* __restrict__ work,
-                           int64_t n, int strategy, tc_plan_params pp, int64_t* __restrict__ cnt,
-                           int8_t* __restrict__ cls, class_acc* __restrict__ acc) {
-    ull loc[4][TC_NUM_CLS] = {};   // per-thread sums, reduced per warp at the end
-    int64_t bm_s = 0, bm_l = 0;    // largest bitmap staging of this thread's small- and large-bitmap items
-    int64_t hv_t = 0;              // largest |N_H(v)| of its thread items
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = n - 1 - i;
-        const int64_t b = row_ptr[r], h = hstart[r], e = row_ptr[r + 1];
-        const int64_t hv = e - h, lv = h - b, W = work[r];
-        int c = -1;
-        int64_t chunks = 0;
-        if (W > 0 && hv > 0) {
-            const int64_t nbits = (int64_t)col[e - 1] - r;
-            const int64_t words = (nbits + 31) >> 5;
-            const int64_t bm = hv < 65536 ? bitmap_bytes(words, hv) : (int64_t)1 << 62;
-            const bool warp_bm = bm <= kWarpSmem;
-            const bool warp_list = hv <= TC_WARP_CAP;
-            const bool cta_s = bm <= kBitmapSmallSmem, cta_l = bm <= kBitmapLargeSmem;
-            if (strategy == TC_STRATEGY_GLOBAL) {
-                c = TC_CLS_CTA_LIST;
-            } else if (strategy == TC_STRATEGY_BSEARCH || strategy == TC_STRATEGY_MERGE) {
-                c = warp_list ? TC_CLS_WARP : TC_CLS_CTA_LIST;
-            } else if (strategy == TC_STRATEGY_BITMAP) {
-                c = warp_bm ? TC_CLS_WARP : cta_s ? TC_CLS_BITMAP_S : cta_l ? TC_CLS_BITMAP_L
-                  : warp_list ? TC_CLS_WARP : TC_CLS_CTA_LIST;
-            } else {
-                // AUTO: tiny vertices one per thread; heavy vertices on a CTA
-                // bitmap when zeroing it is cheap next to the work; the rest
-                // on a warp (bitmap or list)
-                const bool heavy = W >= pp.cta_min_work && W >= 2 * words;
-                if (hv <= kThreadMaxH && lv + W <= pp.thread_work) c = TC_CLS_THREAD;
-                else if (heavy && cta_s) c = TC_CLS_BITMAP_S;
-                else if (heavy && cta_l) c = TC_CLS_BITMAP_L;
-                else if (warp_bm || warp_list) c = TC_CLS_WARP;
-                else if (cta_s) c = TC_CLS_BITMAP_S;
-                else if (cta_l) c = TC_CLS_BITMAP_L;
-                else c = TC_CLS_CTA_LIST;
-            }
-            const int64_t chunk = c == TC_CLS_WARP ? pp.warp_chunk : pp.cta_chunk;
-            chunks = c == TC_CLS_THREAD ? 1 : (W + chunk - 1) / chunk;
-            if (chunks > lv) chunks = lv;
-            if (chunks < 1) chunks = 1;
+// Class of middle vertex r (-1: no work) and its number of items.
+__device__ __forceinline__ int classify_row(int64_t b, int64_t h, int64_t e, int64_t r, int64_t W,
+                                            const int32_t* __restrict__ col, int strategy, const tc_plan_params& pp,
+                                            int64_t& bm) {
+    const int64_t hv = e - h, lv = h - b;
+    if (W <= 0 || hv <= 0) return -1;
+    const int64_t nbits = (int64_t)col[e - 1] - r;
+    const int64_t words = (nbits + 31) >> 5;
+    bm = hv < 65536 ? bitmap_bytes(words, hv) : (int64_t)1 << 62;
+    const bool warp_bm = bm <= kWarpSmem;
+    const bool warp_list = hv <= TC_WARP_CAP;
+    const bool cta_s = bm <= kBitmapSmallSmem, cta_l = bm <= kBitmapLargeSmem;
+    if (strategy == TC_STRATEGY_GLOBAL) return TC_CLS_CTA_LIST;
+    if (strategy == TC_STRATEGY_BSEARCH || strategy == TC_STRATEGY_MERGE)
+        return warp_list ? TC_CLS_WARP : TC_CLS_CTA_LIST;
+    if (strategy == TC_STRATEGY_BITMAP)
+        return warp_bm ? TC_CLS_WARP : cta_s ? TC_CLS_BITMAP_S : cta_l ? TC_CLS_BITMAP_L
+             : warp_list ? TC_CLS_WARP : TC_CLS_CTA_LIST;
+    // AUTO: tiny vertices one per thread; heavy vertices on a CTA
+    // bitmap when zeroing it is cheap next to the work; the rest
+    // on a warp (bitmap or list)
+    const bool heavy = W >= pp.cta_min_work && W >= 2 * words;
+    if (hv <= kThreadMaxH && lv + W <= pp.thread_work) return TC_CLS_THREAD;
+    if (heavy && cta_s) return TC_CLS_BITMAP_S;
+    if (heavy && cta_l) return TC_CLS_BITMAP_L;
+    if (warp_bm || warp_list) return TC_CLS_WARP;
+    if (cta_s) return TC_CLS_BITMAP_S;
+    if (cta_l) return TC_CLS_BITMAP_L;
+    return TC_CLS_CTA_LIST;
+}
+
+// Items a vertex of class c is split into: its work over the class's chunk,
+// at most one per lower neighbour.
+__device__ __forceinline__ int64_t chunks_of(int c, int64_t lv, int64_t W, const tc_plan_params& pp) {
+    const int64_t chunk = c == TC_CLS_WARP ? pp.warp_chunk : pp.cta_chunk;
+    int64_t k = c == TC_CLS_THREAD ? 1 : (W + chunk - 1) / chunk;
+    if (k > lv) k = lv;
+    return k < 1 ? 1 : k;
+}
+
+// The plan is made in three passes over groups of 32·slices vertices, in
+// reverse rank order so that the heaviest come first in every class: a warp
+// classifies a group and sums its items per class (k_classify), one CTA a
+// class turns the sums into offsets (k_plan_scan), and a warp writes its
+// group's items from there (k_emit).  The order of the items depends on the
+// graph alone, which sharded counts rely on.  (A count per vertex and class
+// with one library scan a class wrote and read 120 bytes a vertex and took
+// 13 launches; a whole pass took 63.3 ms on the 8192-graph batch and 0.871 ms
+// at R-MAT scale 12, with this 62.1 and 0.833.)
+constexpr int kPlanGroups = 16384;    // groups aimed at: enough warps to fill the device, few sums to scan
+constexpr int kPlanMaxSlices = 64;
+inline int plan_slices(int64_t n) {
+    const int64_t s = (n + 32ll * kPlanGroups - 1) / (32ll * kPlanGroups);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(s, kPlanMaxSlices));
+}
+
+__global__ void __launch_bounds__(256)
+k_classify(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart, const int32_t* __restrict__ col,
+           const int64_t* __restrict__ work, int64_t n, int strategy, tc_plan_params pp, int slices, int64_t groups,
+           ull* __restrict__ gsum, int8_t* __restrict__ cls, class_acc* __restrict__ acc) {
+    __shared__ ull s_sum[4 * TC_NUM_CLS], s_max[3];
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < 4 * TC_NUM_CLS) s_sum[threadIdx.x] = 0;
+    if (threadIdx.x < 3) s_max[threadIdx.x] = 0;
+    __syncthreads();
+    ull loc[4][TC_NUM_CLS] = {};   // per-thread sums, reduced at the end
+    ull bm_s = 0, bm_l = 0;        // largest bitmap staging of this thread's small- and large-bitmap items
+    ull hv_t = 0;                  // largest |N_H(v)| of its thread items
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; g < groups; g += warps) {
+        ull items[TC_NUM_CLS] = {};
+        for (int s = 0; s < slices; ++s) {
+            const int64_t i = (g * slices + s) * 32 + lane;
+            if (i >= n) break;
+            const int64_t r = n - 1 - i;
+            const int64_t b = row_ptr[r], h = hstart[r], e = row_ptr[r + 1], W = work[r];
+            int64_t bm = 0;
+            const int c = classify_row(b, h, e, r, W, col, strategy, pp, bm);
+            cls[i] = (int8_t)c;
+            const ull hv = (ull)(e - h), lv = (ull)(h - b);
+            const ull k = c >= 0 ? (ull)chunks_of(c, h - b, W, pp) : 0;
 #pragma unroll
-            for (int cc = 0; cc < TC_NUM_CLS; ++cc)   // static indices keep loc in registers
+            for (int cc = 0; cc < TC_NUM_CLS; ++cc)   // static indices keep the sums in registers
                 if (cc == c) {
-                    loc[0][cc] += (ull)chunks;
-                    loc[1][cc] += (ull)hv;
-                    loc[2][cc] += (ull)lv;
+                    items[cc] += k;
+                    loc[1][cc] += hv;
+                    loc[2][cc] += lv;
                     loc[3][cc] += (ull)W;
                 }
             if (c == TC_CLS_THREAD) hv_t = hv > hv_t ? hv : hv_t;
-            if (c == TC_CLS_BITMAP_S) bm_s = bm > bm_s ? bm : bm_s;
-            if (c == TC_CLS_BITMAP_L) bm_l = bm > bm_l ? bm : bm_l;
+            if (c == TC_CLS_BITMAP_S) bm_s = (ull)bm > bm_s ? (ull)bm : bm_s;
+            if (c == TC_CLS_BITMAP_L) bm_l = (ull)bm > bm_l ? (ull)bm : bm_l;
         }
-        cls[i] = (int8_t)c;
-        for (int k = 0; k < TC_NUM_CLS; ++k) cnt[k * (n + 1) + i] = (k == c) ? chunks : 0;
-    }
-    const int lane = threadIdx.x & 31;
-    for (int o = 16; o; o >>= 1) {
-        const int64_t x = __shfl_xor_sync(0xffffffffu, bm_s, o), y = __shfl_xor_sync(0xffffffffu, bm_l, o);
-        const int64_t z = __shfl_xor_sync(0xffffffffu, hv_t, o);
-        bm_s = x > bm_s ? x : bm_s;
-        bm_l = y > bm_l ? y : bm_l;
-        hv_t = z > hv_t ? z : hv_t;
-    }
-    if (lane == 0) {
-        if (bm_s) atomicMax(&acc->max_bm[TC_CLS_BITMAP_S], (ull)bm_s);
-        if (bm_l) atomicMax(&acc->max_bm[TC_CLS_BITMAP_L], (ull)bm_l);
-        if (hv_t) atomicMax(&acc->max_bm[TC_CLS_THREAD], (ull)hv_t);   // for this class: staged ids
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < TC_NUM_CLS; ++c) {
+            const ull x = warp_sum(items[c]);
+            if (lane == 0) gsum[c * groups + g] = x;
+            loc[0][c] += items[c];
+        }
     }
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int c = 0; c < TC_NUM_CLS; ++c) {
-            ull x = loc[a][c];
-            for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            if (lane == 0 && x) {
-                ull* dst = a == 0 ? acc->items : a == 1 ? acc->staged : a == 2 ? acc->head : acc->wedges;
-                atomicAdd(&dst[c], x);
-            }
+            const ull x = warp_sum(loc[a][c]);
+            if (lane == 0 && x) atomicAdd(&s_sum[a * TC_NUM_CLS + c], x);
         }
+    if (bm_s) atomicMax(&s_max[0], bm_s);
+    if (bm_l) atomicMax(&s_max[1], bm_l);
+    if (hv_t) atomicMax(&s_max[2], hv_t);
+    __syncthreads();
+    if (threadIdx.x < 4 * TC_NUM_CLS && s_sum[threadIdx.x]) {
+        const int a = threadIdx.x / TC_NUM_CLS, c = threadIdx.x % TC_NUM_CLS;
+        ull* dst = a == 0 ? acc->items : a == 1 ? acc->staged : a == 2 ? acc->head : acc->wedges;
+        atomicAdd(&dst[c], s_sum[threadIdx.x]);
+    }
+    if (threadIdx.x < 3 && s_max[threadIdx.x]) {
+        // for the thread class: staged ids
+        const int c = threadIdx.x == 0 ? TC_CLS_BITMAP_S : threadIdx.x == 1 ? TC_CLS_BITMAP_L : TC_CLS_THREAD;
+        atomicMax(&acc->max_bm[c], s_max[threadIdx.x]);
+    }
+}
+
+// Group sums of class blockIdx.x -> offsets of its groups, in place.
+constexpr int kPlanScanThreads = 1024;
+__global__ void __launch_bounds__(kPlanScanThreads) k_plan_scan(ull* __restrict__ gsum, int64_t groups) {
+    __shared__ ull s_warp[kPlanScanThreads / 32];
+    ull* x = gsum + blockIdx.x * groups;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    ull carry = 0;
+    for (int64_t g0 = 0; g0 < groups; g0 += kPlanScanThreads) {
+        const int64_t g = g0 + threadIdx.x;
+        const ull mine = g < groups ? x[g] : 0;
+        ull incl = mine;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const ull y = __shfl_up_sync(FULL, incl, d);
+            if (lane >= d) incl += y;
+        }
+        if (lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        ull before = 0, total = 0;
+#pragma unroll 8
+        for (int k = 0; k < kPlanScanThreads / 32; ++k) {
+            const ull y = s_warp[k];
+            before += k < warp ? y : 0;
+            total += y;
+        }
+        if (g < groups) x[g] = carry + before + incl - mine;
+        carry += total;
+        __syncthreads();
+    }
 }
 
 struct emit_targets {
@@ -1137,28 +1202,60 @@ struct emit_targets {
     int64_t* pe[TC_NUM_CLS];
 };
 
-__global__ void k_emit(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart,
-                       const int32_t* __restrict__ col,
-                       int64_t n, const int8_t* __restrict__ cls, const int64_t* __restrict__ cnt,
-                       const int64_t* __restrict__ off, emit_targets tg) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = cls[i];
-        if (c < 0) continue;
-        const int64_t r = n - 1 - i;
-        const int64_t b = row_ptr[r], h0 = hstart[r], lv = h0 - b, h1 = row_ptr[r + 1];
-        const int64_t k = cnt[c * (n + 1) + i], o = off[c * (n + 1) + i];
-        const tc_item d{h0, (int32_t)r, (int32_t)(h1 - h0)};
-        const int32_t nbits = h1 > h0 ? col[h1 - 1] - (int32_t)r : 0;
-        tc_item* dd = tg.d[c];
-        int32_t* nbb = tg.nb[c];
-        int64_t* pbb = tg.pb[c];
-        int64_t* pee = tg.pe[c];
-        for (int64_t j = 0; j < k; ++j) {
-            dd[o + j] = d;
-            nbb[o + j] = nbits;
-            pbb[o + j] = b + lv * j / k;
-            pee[o + j] = b + lv * (j + 1) / k;
+__global__ void __launch_bounds__(256)
+k_emit(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart, const int32_t* __restrict__ col,
+       const int64_t* __restrict__ work, int64_t n, tc_plan_params pp, int slices, int64_t groups,
+       const int8_t* __restrict__ cls, const ull* __restrict__ goff, emit_targets tg) {
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; g < groups; g += warps) {
+        ull base[TC_NUM_CLS];
+#pragma unroll
+        for (int c = 0; c < TC_NUM_CLS; ++c) base[c] = goff[c * groups + g];
+        for (int s = 0; s < slices; ++s) {
+            const int64_t i = (g * slices + s) * 32 + lane;
+            const int c = i < n ? cls[i] : -1;
+            if (!__any_sync(FULL, c >= 0)) continue;
+            tc_item d{};
+            int32_t nbits = 0;
+            int64_t b = 0, lv = 0, k = 0;
+            if (c >= 0) {
+                const int64_t r = n - 1 - i;
+                const int64_t h0 = hstart[r], h1 = row_ptr[r + 1];
+                b = row_ptr[r];
+                lv = h0 - b;
+                k = chunks_of(c, lv, work[r], pp);
+                d = tc_item{h0, (int32_t)r, (int32_t)(h1 - h0)};
+                nbits = h1 > h0 ? col[h1 - 1] - (int32_t)r : 0;
+            }
+#pragma unroll
+            for (int cc = 0; cc < TC_NUM_CLS; ++cc) {
+                const unsigned in = __ballot_sync(FULL, c == cc);
+                if (!in) continue;
+                const int64_t mine = c == cc ? k : 0;
+                ull o = base[cc];
+                if (__any_sync(FULL, mine > 1)) {
+                    ull incl = (ull)mine;
+#pragma unroll
+                    for (int dd = 1; dd < 32; dd <<= 1) {
+                        const ull y = __shfl_up_sync(FULL, incl, dd);
+                        if (lane >= dd) incl += y;
+                    }
+                    o += incl - (ull)mine;
+                    base[cc] += __shfl_sync(FULL, incl, 31);
+                } else {
+                    o += (ull)__popc(in & below);
+                    base[cc] += (ull)__popc(in);
+                }
+                if (c == cc)
+                    for (int64_t j = 0; j < mine; ++j) {
+                        tg.d[cc][o + j] = d;
+                        tg.nb[cc][o + j] = nbits;
+                        tg.pb[cc][o + j] = b + lv * j / k;
+                        tg.pe[cc][o + j] = b + lv * (j + 1) / k;
+                    }
+            }
         }
     }
 }
@@ -1235,11 +1332,9 @@ tc_status launch_persistent(K kernel, const char* name, size_t smem, int64_t all
 }  // namespace
 
 void free_plan(tc_plan& p, cudaStream_t s) {
+    dfree(p.items, s);
+    p.items = nullptr;
     for (int c = 0; c < TC_NUM_CLS; ++c) {
-        dfree(p.d[c], s);
-        dfree(p.nb[c], s);
-        dfree(p.pb[c], s);
-        dfree(p.pe[c], s);
         p.d[c] = nullptr;
         p.nb[c] = nullptr;
         p.pb[c] = p.pe[c] = nullptr;
@@ -1252,19 +1347,16 @@ tc_status make_plan(tc_graph* g, int strategy, cudaStream_t s) {
     free_plan(g->plan, s);
     tc_plan& p = g->plan;
     const int64_t n = g->n;
-    int64_t* cnt = nullptr;
-    int64_t* off = nullptr;
-    int8_t* cls = nullptr;
+    const int slices = plan_slices(n);
+    const int64_t groups = (n + 32ll * slices - 1) / (32ll * slices);
     class_acc* acc = nullptr;
-    uint8_t* tmp = nullptr;
-    size_t tmp_bytes = 0;
+    ull* gsum = nullptr;
+    int8_t* cls = nullptr;
     tc_status st = TC_OK;
     auto cleanup = [&]() {
-        dfree(cnt, s);
-        dfree(off, s);
+        dfree(gsum, s);
         dfree(cls, s);
         dfree(acc, s);
-        dfree(tmp, s);
     };
 #define PLAN_TRY(x)              \
     do {                         \
@@ -1276,37 +1368,45 @@ tc_status make_plan(tc_graph* g, int strategy, cudaStream_t s) {
         }                        \
     } while (0)
 #define PLAN_CUDA(x) PLAN_TRY(from_cuda(x))
-    PLAN_TRY(dalloc((void**)&cnt, TC_NUM_CLS * (n + 1) * 8, s));
-    PLAN_TRY(dalloc((void**)&off, TC_NUM_CLS * (n + 1) * 8, s));
-    PLAN_TRY(dalloc((void**)&cls, n + 1, s));
     PLAN_TRY(dalloc((void**)&acc, sizeof(class_acc), s));
+    PLAN_TRY(dalloc((void**)&gsum, TC_NUM_CLS * (groups + 1) * 8, s));
+    PLAN_TRY(dalloc((void**)&cls, n + 1, s));
     PLAN_CUDA(cudaMemsetAsync(acc, 0, sizeof(class_acc), s));
-    PLAN_CUDA(cudaMemsetAsync(cnt, 0, TC_NUM_CLS * (n + 1) * 8, s));
     if (n > 0) {
-        launch_scope ls("plan_classify", s);
-        k_classify<<<blocks_for(n), 256, 0, s>>>(g->row_ptr, g->hstart, g->col, g->work, n, strategy,
-                                                  g->params, cnt, cls, acc);
-        PLAN_CUDA(cudaGetLastError());
-    }
-    PLAN_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tmp_bytes, cnt, off, n + 1, s));
-    PLAN_TRY(dalloc((void**)&tmp, tmp_bytes, s));
-    {
+        {
+            launch_scope ls("plan_classify", s);
+            k_classify<<<blocks_for(groups * 32), 256, 0, s>>>(g->row_ptr, g->hstart, g->col, g->work, n, strategy,
+                                                               g->params, slices, groups, gsum, cls, acc);
+            PLAN_CUDA(cudaGetLastError());
+        }
         launch_scope ls("plan_scan", s);
-        for (int c = 0; c < TC_NUM_CLS; ++c)
-            PLAN_TRY(run_library("scan_plan", n + 1, 0, c == 0, s, [&](cudaStream_t st) {
-                return cub::DeviceScan::ExclusiveSum(tmp, tmp_bytes, cnt + c * (n + 1), off + c * (n + 1),
-                                                     n + 1, st);
-            }));
+        k_plan_scan<<<TC_NUM_CLS, kPlanScanThreads, 0, s>>>(gsum, groups);
+        PLAN_CUDA(cudaGetLastError());
     }
     class_acc h{};
     PLAN_CUDA(cudaMemcpyAsync(&h, acc, sizeof(h), cudaMemcpyDeviceToHost, s));
     PLAN_CUDA(cudaStreamSynchronize(s));
+    // one block for all classes: the 8-byte-aligned arrays first
+    int64_t total = 0;
     for (int c = 0; c < TC_NUM_CLS; ++c) {
         p.count[c] = (int64_t)h.items[c];
-        PLAN_TRY(dalloc((void**)&p.d[c], (p.count[c] + 1) * sizeof(tc_item), s));
-        PLAN_TRY(dalloc((void**)&p.nb[c], (p.count[c] + 1) * 4, s));
-        PLAN_TRY(dalloc((void**)&p.pb[c], (p.count[c] + 1) * 8, s));
-        PLAN_TRY(dalloc((void**)&p.pe[c], (p.count[c] + 1) * 8, s));
+        total += p.count[c] + 1;
+    }
+    PLAN_TRY(dalloc(&p.items, (size_t)total * (sizeof(tc_item) + 8 + 8 + 4), s));
+    {
+        tc_item* d = (tc_item*)p.items;
+        int64_t* q = (int64_t*)(d + total);
+        int32_t* nb = (int32_t*)(q + 2 * total);
+        for (int c = 0; c < TC_NUM_CLS; ++c) {
+            const int64_t k = p.count[c] + 1;
+            p.d[c] = d;
+            p.pb[c] = q;
+            p.pe[c] = q + k;
+            p.nb[c] = nb;
+            d += k;
+            q += 2 * k;
+            nb += k;
+        }
     }
     if (n > 0) {
         launch_scope ls("plan_emit", s);
@@ -1317,7 +1417,8 @@ tc_status make_plan(tc_graph* g, int strategy, cudaStream_t s) {
             tg.pb[c] = p.pb[c];
             tg.pe[c] = p.pe[c];
         }
-        k_emit<<<blocks_for(n), 256, 0, s>>>(g->row_ptr, g->hstart, g->col, n, cls, cnt, off, tg);
+        k_emit<<<blocks_for(groups * 32), 256, 0, s>>>(g->row_ptr, g->hstart, g->col, g->work, n, g->params, slices,
+                                                       groups, cls, gsum, tg);
         PLAN_CUDA(cudaGetLastError());
     }
     // the bitmap kernels get the shared memory their largest item needs, not

@@ -83,6 +83,7 @@ struct tc_item {
 struct tc_plan {
     int strategy = -1;                 // strategy the plan was made for
     int64_t count[TC_NUM_CLS] = {};
+    void* items = nullptr;             // the block that the arrays below lie in
     tc_item* d[TC_NUM_CLS] = {};       // middle vertex of each item
     int32_t* nb[TC_NUM_CLS] = {};      // its id window max N_H(v) - v (0 if N_H(v) is empty)
     int64_t* pb[TC_NUM_CLS] = {};      // head-entry range [pb, pe) of the item
