@@ -975,22 +975,42 @@ k_count_thread(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ 
         }
         ull tv = 0;
         const int64_t pb = it_pb[gi], pe = it_pe[gi];
-        tc_head nrec{};
-        if (pb < pe) nrec = head[TC_IX(pb, dm.e2)];
+        // head records two ahead and the first ids of the next stream are in
+        // flight while a stream is merged, so a thread does not wait for a
+        // record and then for its stream in turn
+        tc_head rec{}, nrec{};
+        int32_t first[kThreadILP];
+        auto fetch_first = [&](const tc_head& r) {
+#pragma unroll
+            for (int j = 0; j < kThreadILP; ++j)
+                first[j] = j < r.hrem ? col[TC_IX(r.twin + 1 + j, dm.e2)] : 0;
+        };
+        if (pb < pe) {
+            nrec = head[TC_IX(pb, dm.e2)];
+            fetch_first(nrec);
+            rec = nrec;
+            if (pb + 1 < pe) nrec = head[TC_IX(pb + 1, dm.e2)];
+        }
         for (int64_t p = pb; p < pe; ++p) {
-            const tc_head rec = nrec;
-            if (p + 1 < pe) nrec = head[TC_IX(p + 1, dm.e2)];   // in flight meanwhile
             const int64_t q0 = rec.twin + 1;
             const int len = rec.hrem;
+            const int32_t u = rec.u;
+            int32_t wv[kThreadILP];
+#pragma unroll
+            for (int j = 0; j < kThreadILP; ++j) wv[j] = first[j];
+            if (p + 1 < pe) {
+                rec = nrec;
+                fetch_first(rec);
+                if (p + 2 < pe) nrec = head[TC_IX(p + 2, dm.e2)];
+            }
             uint32_t hits = 0;
             // first staged id not below the stream's first id (bisection)
             int a = 0;
             if (len > 0) {
-                const int32_t w0 = col[TC_IX(q0, dm.e2)];
                 int cnt = hv;
                 while (cnt > 0) {
                     const int half = cnt >> 1;
-                    if (S[a + half][t] < w0) {
+                    if (S[a + half][t] < wv[0]) {
                         a += half + 1;
                         cnt -= half + 1;
                     } else {
@@ -999,9 +1019,10 @@ k_count_thread(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ 
                 }
             }
             for (int j0 = 0; j0 < len && a < hv; j0 += kThreadILP) {
-                int32_t wv[kThreadILP];
+                if (j0 > 0) {
 #pragma unroll
-                for (int j = 0; j < kThreadILP; ++j) wv[j] = j0 + j < len ? col[TC_IX(q0 + j0 + j, dm.e2)] : 0;
+                    for (int j = 0; j < kThreadILP; ++j) wv[j] = j0 + j < len ? col[TC_IX(q0 + j0 + j, dm.e2)] : 0;
+                }
 #pragma unroll
                 for (int j = 0; j < kThreadILP; ++j) {
                     const int32_t w = wv[j];
@@ -1018,8 +1039,8 @@ k_count_thread(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ 
                 }
             }
             if (hits) {
-                atomicAdd(&tri[TC_IX(rec.u, dm.n)], (ull)hits);
-                mark<EC>(flag, rec.twin, hits, dm);
+                atomicAdd(&tri[TC_IX(u, dm.n)], (ull)hits);
+                mark<EC>(flag, q0 - 1, hits, dm);
                 tv += hits;
             }
         }
