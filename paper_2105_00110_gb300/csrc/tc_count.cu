@@ -661,6 +661,9 @@ struct warp_smem {
     uint32_t filt[kFilterWords];
     stream_table<32> tb;
 };
+// Items a warp takes from the queue at a time: four where there are many
+// (fewer atomics), one where four would leave warps without any (706 items
+// at R-MAT scale 12 were 177 warps with four each: 147 us).
 #ifndef TC_WARP_FETCH
 #define TC_WARP_FETCH 4
 #endif
@@ -717,12 +720,13 @@ k_count_warp(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ co
     const bool allow_bitmap = !MERGE && (strategy == TC_STRATEGY_AUTO || strategy == TC_STRATEGY_BITMAP);
     ull tv_all = 0;
     auto wbar = [] { __syncwarp(); };
+    const int fetch = n_items >= 8ll * kWarpItemsPerFetch * kCtaWarps * gridDim.x ? kWarpItemsPerFetch : 1;
     for (;;) {
         int64_t base = 0;
-        if (lane == 0) base = (int64_t)atomicAdd(cursor, (ull)kWarpItemsPerFetch);
+        if (lane == 0) base = (int64_t)atomicAdd(cursor, (ull)fetch);
         base = __shfl_sync(FULL, base, 0);
         if (base >= n_items) break;
-        const int64_t lim = min(base + kWarpItemsPerFetch, n_items);
+        const int64_t lim = min(base + fetch, n_items);
         for (int64_t it = base; it < lim; ++it) {
             const int64_t gi = it_off + it_stride * it;   // this shard's it-th item
             const tc_item d = it_d[gi];
