@@ -1071,8 +1071,11 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
     // Unions of many small graphs hold millions of light vertices; one
     // thread each for those of up to 128 ids of work instead of 64 (the
     // 8192-graph batch: count 7.9 -> 6.7 ms; on the grid workload the
-    // larger cap was 0.3 ms slower, so single graphs keep 64).
-    if (flags & TC_BUILD_NO_CORE) g->params.thread_work = 128;
+    // larger cap was 0.3 ms slower, so single graphs keep 64).  With fewer
+    // vertices than keep every thread of the device busy several times over,
+    // the longest thread item alone sets that kernel's time: the cap is 16.
+    if (n < (int64_t)sm_count() * 2048 * 4) g->params.thread_work = 16;
+    else if (flags & TC_BUILD_NO_CORE) g->params.thread_work = 128;
     TC_TRY(make_plan(g, g->strategy, s));
     TC_CUDA(cudaStreamSynchronize(s));
     return TC_OK;

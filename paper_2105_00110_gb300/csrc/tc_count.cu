@@ -714,6 +714,7 @@ k_count_warp(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ co
              const int64_t* __restrict__ it_pb, const int64_t* __restrict__ it_pe,
              int64_t n_items, int64_t it_off, int64_t it_stride, ull* __restrict__ cursor, int strategy,
              ull* __restrict__ tri, uint32_t* __restrict__ flag, ull* __restrict__ total, tc_dims dm) {
+    pdl_trigger();
     __shared__ __align__(16) warp_smem sm[kCtaWarps];
     const int lane = threadIdx.x & 31;
     warp_smem& ws = sm[threadIdx.x >> 5];
@@ -794,6 +795,7 @@ k_count_warp(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ co
         }
     }
     if (lane == 0 && tv_all) atomicAdd(total, tv_all);
+    pdl_wait();
 }
 
 // ------------------------------------------------------------- CTA items
@@ -812,6 +814,7 @@ k_count_cta(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col
             int64_t n_items, int64_t it_off, int64_t it_stride, ull* __restrict__ cursor, int strategy,
             ull* __restrict__ tri,
             uint32_t* __restrict__ flag, ull* __restrict__ total, tc_dims dm) {
+    pdl_trigger();
     extern __shared__ __align__(16) uint8_t dyn[];
     __shared__ __align__(16) stream_table<T> tb;
     __shared__ int64_t s_item;
@@ -920,6 +923,7 @@ k_count_cta(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col
             }
         }
     }
+    pdl_wait();
 }
 
 // ------------------------------------------------------------ thread items
@@ -957,6 +961,7 @@ k_count_thread(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ 
                const int64_t* __restrict__ it_pe, int64_t n_items, int64_t it_off, int64_t it_stride,
                ull* __restrict__ cursor, int strategy,
                ull* __restrict__ tri, uint32_t* __restrict__ flag, ull* __restrict__ total, tc_dims dm) {
+    pdl_trigger();
     __shared__ int32_t S[MAXH][kThreadBlock];   // items with MINH <= |N_H(v)| <= MAXH; the others skipped
     const int t = threadIdx.x;
     ull tv_all = 0;
@@ -1053,6 +1058,7 @@ k_count_thread(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ 
     }
     tv_all = warp_sum(tv_all);
     if ((t & 31) == 0 && tv_all) atomicAdd(total, tv_all);
+    pdl_wait();
 }
 
 // ------------------------------------------------------------ planner
@@ -1334,10 +1340,17 @@ tc_status shape_for(const void* fn, size_t smem, int threads, int& per_sm) {
     return TC_OK;
 }
 
+// The class kernels of one count are independent of each other (they only
+// add to tri, the marks and the total), so all but the first are launched to
+// start as the CTAs of the one before run out of items, instead of after its
+// last: each lets the next be set up from its start and waits at its end
+// until the one before has finished, so that the last one's end is the end
+// of all.  `first`: the kernel after the clears, which starts when they are
+// done.
 template <class K>
 tc_status launch_persistent(K kernel, const char* name, size_t smem, int64_t all_items, cudaStream_t s,
                             const tc_graph* g, const tc_plan& p, int c, ull* cursor, uint32_t* marks,
-                            int shard, int num_shards, int threads = TC_CTA_THREADS) {
+                            int shard, int num_shards, bool& first, int threads = TC_CTA_THREADS) {
     // shard k of K takes items k, k + K, k + 2K, ... of the class (heaviest
     // first, so the shards' work comes out close to equal)
     const int64_t items = all_items > shard ? (all_items - shard + num_shards - 1) / num_shards : 0;
@@ -1346,11 +1359,17 @@ tc_status launch_persistent(K kernel, const char* name, size_t smem, int64_t all
     TC_TRY(shape_for((const void*)kernel, smem, threads, per_sm));
     int64_t blocks = std::min<int64_t>((int64_t)sm_count() * per_sm, items);
     launch_scope ls(name, s);
-    kernel<<<(int)blocks, threads, smem, s>>>(g->row_ptr, g->col, g->hstart, g->head,
-                                                     p.d[c], p.nb[c], p.pb[c], p.pe[c], items, (int64_t)shard,
-                                                     (int64_t)num_shards, cursor,
-                                                     g->strategy, g->tri, marks, g->counters, dims_of(g));
-    TC_LAUNCH_CHECK();
+    if (first) {
+        first = false;
+        kernel<<<(int)blocks, threads, smem, s>>>(g->row_ptr, g->col, g->hstart, g->head, p.d[c], p.nb[c], p.pb[c],
+                                                  p.pe[c], items, (int64_t)shard, (int64_t)num_shards, cursor,
+                                                  g->strategy, g->tri, marks, g->counters, dims_of(g));
+        TC_LAUNCH_CHECK();
+    } else {
+        TC_CUDA(launch_pdl(kernel, (int)blocks, threads, smem, s, g->row_ptr, g->col, g->hstart, g->head, p.d[c],
+                           p.nb[c], p.pb[c], p.pe[c], items, (int64_t)shard, (int64_t)num_shards, cursor, g->strategy,
+                           g->tri, marks, g->counters, dims_of(g)));
+    }
     return TC_OK;
 }
 
@@ -1497,6 +1516,7 @@ tc_status launch_count_kernels(tc_graph* g, cudaStream_t s, uint32_t* marks, int
     const tc_plan& p = g->plan;
     ull* cur = g->counters + 1;
     const bool merge = g->strategy == TC_STRATEGY_MERGE;
+    bool first = true;
     const char* nm[5] = {EC ? "count_edges_bitmap_l" : "count_bitmap_l", EC ? "count_edges_bitmap_s" : "count_bitmap_s",
                          EC ? "count_edges_cta_list" : "count_cta_list", EC ? "count_edges_cta_global" : "count_cta_global",
                          EC ? "count_edges_warp" : "count_warp"};
@@ -1505,29 +1525,30 @@ tc_status launch_count_kernels(tc_graph* g, cudaStream_t s, uint32_t* marks, int
     // 16 ids) run those in a launch that holds half of it, the rest going
     // to L1, and the others, if any, in a second launch over the same list
     // (the 8192-graph batch: 5.0 -> 3.9 ms); with fewer items the second
-    // pass over the list costs more than it saves
+    // pass over the list costs more than it saves.  They come first: a
+    // kernel that starts beside another on an SM gets the L1 that one left
+    // (after the warp kernel the batch's thread items took 1 ms longer)
     const bool split = p.thread_max_h <= 16 || p.count[TC_CLS_THREAD] >= kThreadSplitItems;
     if (split)
         TC_TRY(launch_persistent(k_count_thread<EC, 16, 0>, EC ? "count_edges_thread" : "count_thread", 0,
-                                 p.count[TC_CLS_THREAD], s, g, p, TC_CLS_THREAD, cur + TC_CLS_THREAD, marks, shard,
-                                 num_shards, kThreadBlock));
+                                 p.count[TC_CLS_THREAD], s, g, p, TC_CLS_THREAD, cur + TC_CLS_THREAD, marks, shard, num_shards, first, kThreadBlock));
     if (split && p.thread_max_h > 16)
         TC_TRY(launch_persistent(k_count_thread<EC, kThreadMaxH, 17>, EC ? "count_edges_thread" : "count_thread",
                                  0, p.count[TC_CLS_THREAD], s, g, p, TC_CLS_THREAD, cur + TC_CLS_THREAD, marks,
-                                 shard, num_shards, kThreadBlock));
+                                 shard, num_shards, first, kThreadBlock));
     else if (!split)
         TC_TRY(launch_persistent(k_count_thread<EC, kThreadMaxH, 0>, EC ? "count_edges_thread" : "count_thread",
                                  0, p.count[TC_CLS_THREAD], s, g, p, TC_CLS_THREAD, cur + TC_CLS_THREAD, marks,
-                                 shard, num_shards, kThreadBlock));
+                                 shard, num_shards, first, kThreadBlock));
     // heaviest classes first; each kernel drains its own item queue
     if (TC_WIDE_L)
         TC_TRY(launch_persistent(k_count_cta<L_BITMAP, false, EC, 2 * kCtaT>, nm[0], p.smem[TC_CLS_BITMAP_L],
                                  p.count[TC_CLS_BITMAP_L], s, g, p, TC_CLS_BITMAP_L, cur + TC_CLS_BITMAP_L, marks,
-                                 shard, num_shards, 2 * kCtaT));
+                                 shard, num_shards, first, 2 * kCtaT));
     else
         TC_TRY(launch_persistent(k_count_cta<L_BITMAP, false, EC>, nm[0], p.smem[TC_CLS_BITMAP_L],
                                  p.count[TC_CLS_BITMAP_L], s, g, p, TC_CLS_BITMAP_L, cur + TC_CLS_BITMAP_L, marks,
-                                 shard, num_shards, kCtaT));
+                                 shard, num_shards, first, kCtaT));
     // small CTA items (grids with Chung-Lu hubs: 2^16-wedge chunks) share
     // their staging and rounds over 16 warps (the 4096^2 grid's bitmap
     // kernel 2.17 -> 1.47 ms); R-MAT's larger items keep 8 (16 were 20 %
@@ -1535,11 +1556,11 @@ tc_status launch_count_kernels(tc_graph* g, cudaStream_t s, uint32_t* marks, int
     if (g->params.cta_chunk < kWideCtaChunk)
         TC_TRY(launch_persistent(k_count_cta<L_BITMAP, false, EC, 2 * kCtaT>, nm[1], p.smem[TC_CLS_BITMAP_S],
                                  p.count[TC_CLS_BITMAP_S], s, g, p, TC_CLS_BITMAP_S, cur + TC_CLS_BITMAP_S, marks,
-                                 shard, num_shards, 2 * kCtaT));
+                                 shard, num_shards, first, 2 * kCtaT));
     else
         TC_TRY(launch_persistent(k_count_cta<L_BITMAP, false, EC>, nm[1], p.smem[TC_CLS_BITMAP_S],
                                  p.count[TC_CLS_BITMAP_S], s, g, p, TC_CLS_BITMAP_S, cur + TC_CLS_BITMAP_S, marks,
-                                 shard, num_shards, kCtaT));
+                                 shard, num_shards, first, kCtaT));
     if (p.count[TC_CLS_CTA_LIST] > 0) {
         // lists longer than the shared budget are searched in place
         const bool fits = g->strategy != TC_STRATEGY_GLOBAL &&
@@ -1547,21 +1568,21 @@ tc_status launch_count_kernels(tc_graph* g, cudaStream_t s, uint32_t* marks, int
         if (fits && merge)
             TC_TRY(launch_persistent(k_count_cta<L_SORTED, true, EC>, nm[2], p.smem[TC_CLS_CTA_LIST],
                                      p.count[TC_CLS_CTA_LIST], s, g, p, TC_CLS_CTA_LIST, cur + TC_CLS_CTA_LIST,
-                                     marks, shard, num_shards, kCtaT));
+                                     marks, shard, num_shards, first, kCtaT));
         else if (fits)
             TC_TRY(launch_persistent(k_count_cta<L_SORTED, false, EC>, nm[2], p.smem[TC_CLS_CTA_LIST],
                                      p.count[TC_CLS_CTA_LIST], s, g, p, TC_CLS_CTA_LIST, cur + TC_CLS_CTA_LIST,
-                                     marks, shard, num_shards, kCtaT));
+                                     marks, shard, num_shards, first, kCtaT));
         else
             TC_TRY(launch_persistent(k_count_cta<L_GLOBAL, false, EC>, nm[3], 0, p.count[TC_CLS_CTA_LIST], s, g,
-                                     p, TC_CLS_CTA_LIST, cur + TC_CLS_CTA_LIST, marks, shard, num_shards, kCtaT));
+                                     p, TC_CLS_CTA_LIST, cur + TC_CLS_CTA_LIST, marks, shard, num_shards, first, kCtaT));
     }
     if (merge)
         TC_TRY(launch_persistent(k_count_warp<true, EC>, nm[4], 0, p.count[TC_CLS_WARP], s, g, p, TC_CLS_WARP,
-                                 cur + TC_CLS_WARP, marks, shard, num_shards));
+                                 cur + TC_CLS_WARP, marks, shard, num_shards, first));
     else
         TC_TRY(launch_persistent(k_count_warp<false, EC>, nm[4], 0, p.count[TC_CLS_WARP], s, g, p, TC_CLS_WARP,
-                                 cur + TC_CLS_WARP, marks, shard, num_shards));
+                                 cur + TC_CLS_WARP, marks, shard, num_shards, first));
     return TC_OK;
 }
 
