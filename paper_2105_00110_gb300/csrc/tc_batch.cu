@@ -39,47 +39,6 @@ inline int blocks(int64_t items) {
     return (int)std::max<int64_t>(1, std::min(b, cap));
 }
 
-// Pairs of graph k (pairs [poff[k], poff[k+1])) -> union labels; an id
-// outside [0, n_k) sets the error word.
-template <typename T>
-__global__ void k_shift_pairs(const T* __restrict__ src, const T* __restrict__ dst, int64_t np,
-                              const int64_t* __restrict__ poff, const int64_t* __restrict__ voff,
-                              int64_t G, int32_t* __restrict__ gs, int32_t* __restrict__ gd,
-                              unsigned int* __restrict__ err) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t lo = 0, hi = G;   // last k with poff[k] <= i
-        while (hi - lo > 1) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (poff[mid] <= i) lo = mid; else hi = mid;
-        }
-        const int64_t nk = voff[lo + 1] - voff[lo];
-        const int64_t a = (int64_t)src[i], b = (int64_t)dst[i];
-        if (a < 0 || b < 0 || a >= nk || b >= nk) {
-            atomicOr(err, 1u);
-            gs[i] = gd[i] = 0;
-        } else {
-            gs[i] = (int32_t)(voff[lo] + a);
-            gd[i] = (int32_t)(voff[lo] + b);
-        }
-    }
-}
-
-// graph of every rank (through its union label)
-__global__ void k_rank_graph(const int32_t* __restrict__ perm, int64_t n, const int64_t* __restrict__ voff,
-                             int64_t G, int32_t* __restrict__ rg) {
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n;
-         r += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t v = perm[r];
-        int64_t lo = 0, hi = G;
-        while (hi - lo > 1) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (voff[mid] <= v) lo = mid; else hi = mid;
-        }
-        rg[r] = (int32_t)lo;
-    }
-}
-
 // first canonical edge of every graph (edges are sorted by union label)
 __global__ void k_edge_offsets(const int32_t* __restrict__ eu, int64_t m, const int64_t* __restrict__ voff,
                                int64_t G, int64_t* __restrict__ eoff) {
@@ -164,43 +123,16 @@ tc_status build_batch(tc_batch* b, const void* src, const void* dst, const int64
         dsrc = a;
         ddst = c;
     }
-    int32_t *gs = nullptr, *gd = nullptr;
-    unsigned int* err = nullptr;
-    B_TRY(get((void**)&gs, (np + 1) * 4));
-    B_TRY(get((void**)&gd, (np + 1) * 4));
-    B_TRY(get((void**)&err, 4));
-    B_TRY(from_cuda(cudaMemsetAsync(err, 0, 4, s)));
-    if (np > 0) {
-        launch_scope ls("batch_shift_pairs", s);
-        if (i32)
-            k_shift_pairs<int32_t><<<blocks(np), 256, 0, s>>>((const int32_t*)dsrc, (const int32_t*)ddst, np,
-                                                              poff, b->voff, G, gs, gd, err);
-        else
-            k_shift_pairs<int64_t><<<blocks(np), 256, 0, s>>>((const int64_t*)dsrc, (const int64_t*)ddst, np,
-                                                              poff, b->voff, G, gs, gd, err);
-        B_TRY(from_cuda(cudaGetLastError()));
-    }
-    unsigned int h_err = 0;
-    B_TRY(from_cuda(cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, s)));
-    B_TRY(from_cuda(cudaStreamSynchronize(s)));
-    if (h_err) {
-        cleanup();
-        return TC_ERR_INVALID_ARG;
-    }
     b->g = new (std::nothrow) tc_graph();
     if (!b->g) {
         cleanup();
         return TC_ERR_OUT_OF_MEMORY;
     }
     cudaGetDevice(&b->g->device);
-    B_TRY(build_graph(b->g, gs, gd, np, n, TC_IN_DEVICE | TC_IDS_INT32 | TC_BUILD_NO_CORE, s));
-    tc_graph* g = b->g;
     B_TRY(dalloc((void**)&b->rank_graph, (n + 1) * 4, s));
-    if (n > 0) {
-        launch_scope ls("batch_rank_graph", s);
-        k_rank_graph<<<blocks(n), 256, 0, s>>>(g->perm, n, b->voff, G, b->rank_graph);
-        B_TRY(from_cuda(cudaGetLastError()));
-    }
+    const union_layout un{poff, b->voff, G, G ? *std::max_element(h_nv, h_nv + G) : 0, b->rank_graph};
+    B_TRY(build_graph(b->g, dsrc, ddst, np, n, TC_IN_DEVICE | (flags & TC_IDS_INT32) | TC_BUILD_NO_CORE, s, &un));
+    tc_graph* g = b->g;
     {
         launch_scope ls("batch_edge_offsets", s);
         k_edge_offsets<<<blocks(G + 1), 256, 0, s>>>(g->edge_u, g->m, b->voff, G, b->eoff);

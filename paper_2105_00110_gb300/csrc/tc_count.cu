@@ -1111,11 +1111,29 @@ __device__ __forceinline__ int64_t chunks_of(int c, int64_t lv, int64_t W, const
     return k < 1 ? 1 : k;
 }
 
+// Items of a class lie by size, the heaviest first, so that the last to run
+// are short and the lanes of a warp of thread items have like work: the warp
+// and thread classes are split into steps of work (order classes; one vertex
+// has one).  Within a step items keep reverse rank order.
+constexpr int kWarpSteps = 3, kThreadSteps = 4;
+constexpr int kNumOrd = 3 + kWarpSteps + kThreadSteps;
+// order classes in the order of enum tc_item_class
+constexpr int kOrdWarp = 2, kOrdList = kOrdWarp + kWarpSteps, kOrdThread = kOrdList + 1;
+__device__ __forceinline__ int order_of(int c, int64_t lv, int64_t W) {
+    if (c <= TC_CLS_BITMAP_L) return c;
+    if (c == TC_CLS_CTA_LIST) return kOrdList;
+    const int64_t x = lv + W;
+    if (c == TC_CLS_WARP) return kOrdWarp + (x > 4096 ? 0 : x > 512 ? 1 : 2);
+    return kOrdThread + (x > 64 ? 0 : x > 24 ? 1 : x > 8 ? 2 : 3);
+}
+__device__ __forceinline__ int class_of_order(int o) {
+    return o < kOrdWarp ? o : o < kOrdList ? TC_CLS_WARP : o == kOrdList ? TC_CLS_CTA_LIST : TC_CLS_THREAD;
+}
+
 // The plan is made in three passes over groups of 32·slices vertices, in
-// reverse rank order so that the heaviest come first in every class: a warp
-// classifies a group and sums its items per class (k_classify), one CTA a
-// class turns the sums into offsets (k_plan_scan), and a warp writes its
-// group's items from there (k_emit).  The order of the items depends on the
+// reverse rank order: a warp classifies a group and sums its items per order
+// class (k_classify), one CTA an order class turns the sums into offsets
+// (k_plan_scan), and a warp writes its group's items from there (k_emit).  The order of the items depends on the
 // graph alone, which sharded counts rely on.  (A count per vertex and class
 // with one library scan a class wrote and read 120 bytes a vertex and took
 // 13 launches; a whole pass took 63.3 ms on the 8192-graph batch and 0.871 ms
@@ -1141,7 +1159,7 @@ k_classify(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hsta
     ull hv_t = 0;                  // largest |N_H(v)| of its thread items
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; g < groups; g += warps) {
-        ull items[TC_NUM_CLS] = {};
+        ull items[kNumOrd] = {};
         for (int s = 0; s < slices; ++s) {
             const int64_t i = (g * slices + s) * 32 + lane;
             if (i >= n) break;
@@ -1149,27 +1167,30 @@ k_classify(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hsta
             const int64_t b = row_ptr[r], h = hstart[r], e = row_ptr[r + 1], W = work[r];
             int64_t bm = 0;
             const int c = classify_row(b, h, e, r, W, col, strategy, pp, bm);
-            cls[i] = (int8_t)c;
+            const int ord = c >= 0 ? order_of(c, h - b, W) : -1;
+            cls[i] = (int8_t)ord;
             const ull hv = (ull)(e - h), lv = (ull)(h - b);
             const ull k = c >= 0 ? (ull)chunks_of(c, h - b, W, pp) : 0;
 #pragma unroll
             for (int cc = 0; cc < TC_NUM_CLS; ++cc)   // static indices keep the sums in registers
                 if (cc == c) {
-                    items[cc] += k;
+                    loc[0][cc] += k;
                     loc[1][cc] += hv;
                     loc[2][cc] += lv;
                     loc[3][cc] += (ull)W;
                 }
+#pragma unroll
+            for (int o = 0; o < kNumOrd; ++o)
+                if (o == ord) items[o] += k;
             if (c == TC_CLS_THREAD) hv_t = hv > hv_t ? hv : hv_t;
             if (c == TC_CLS_BITMAP_S) bm_s = (ull)bm > bm_s ? (ull)bm : bm_s;
             if (c == TC_CLS_BITMAP_L) bm_l = (ull)bm > bm_l ? (ull)bm : bm_l;
         }
         __syncwarp();
 #pragma unroll
-        for (int c = 0; c < TC_NUM_CLS; ++c) {
-            const ull x = warp_sum(items[c]);
-            if (lane == 0) gsum[c * groups + g] = x;
-            loc[0][c] += items[c];
+        for (int o = 0; o < kNumOrd; ++o) {
+            const ull x = warp_sum(items[o]);
+            if (lane == 0) gsum[o * groups + g] = x;
         }
     }
 #pragma unroll
@@ -1195,9 +1216,10 @@ k_classify(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hsta
     }
 }
 
-// Group sums of class blockIdx.x -> offsets of its groups, in place.
+// Group sums of order class blockIdx.x -> offsets of its groups within it, in
+// place; its total into tot.
 constexpr int kPlanScanThreads = 1024;
-__global__ void __launch_bounds__(kPlanScanThreads) k_plan_scan(ull* __restrict__ gsum, int64_t groups) {
+__global__ void __launch_bounds__(kPlanScanThreads) k_plan_scan(ull* __restrict__ gsum, int64_t groups, ull* __restrict__ tot) {
     __shared__ ull s_warp[kPlanScanThreads / 32];
     ull* x = gsum + blockIdx.x * groups;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1224,6 +1246,7 @@ __global__ void __launch_bounds__(kPlanScanThreads) k_plan_scan(ull* __restrict_
         carry += total;
         __syncthreads();
     }
+    if (threadIdx.x == 0) tot[blockIdx.x] = carry;
 }
 
 struct emit_targets {
@@ -1236,56 +1259,63 @@ struct emit_targets {
 __global__ void __launch_bounds__(256)
 k_emit(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart, const int32_t* __restrict__ col,
        const int64_t* __restrict__ work, int64_t n, tc_plan_params pp, int slices, int64_t groups,
-       const int8_t* __restrict__ cls, const ull* __restrict__ goff, emit_targets tg) {
+       const int8_t* __restrict__ cls, const ull* __restrict__ goff, const ull* __restrict__ tot, emit_targets tg) {
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    // first item of each order class in its class's arrays: the steps before it
+    ull start = 0;
+    if (lane < kNumOrd)
+        for (int o = lane - 1; o >= 0 && class_of_order(o) == class_of_order(lane); --o) start += tot[o];
     for (int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; g < groups; g += warps) {
-        ull base[TC_NUM_CLS];
-#pragma unroll
-        for (int c = 0; c < TC_NUM_CLS; ++c) base[c] = goff[c * groups + g];
+        ull off = lane < kNumOrd ? start + goff[lane * groups + g] : 0;
         for (int s = 0; s < slices; ++s) {
             const int64_t i = (g * slices + s) * 32 + lane;
-            const int c = i < n ? cls[i] : -1;
-            if (!__any_sync(FULL, c >= 0)) continue;
-            tc_item d{};
-            int32_t nbits = 0;
-            int64_t b = 0, lv = 0, k = 0;
-            if (c >= 0) {
-                const int64_t r = n - 1 - i;
-                const int64_t h0 = hstart[r], h1 = row_ptr[r + 1];
+            const int ord = i < n ? cls[i] : -1;
+            if (!__any_sync(FULL, ord >= 0)) continue;
+            int64_t b = 0, lv = 0, k = 0, h0 = 0, h1 = 0;
+            const int64_t r = n - 1 - i;
+            if (ord >= 0) {
+                h0 = hstart[r];
+                h1 = row_ptr[r + 1];
                 b = row_ptr[r];
                 lv = h0 - b;
-                k = chunks_of(c, lv, work[r], pp);
-                d = tc_item{h0, (int32_t)r, (int32_t)(h1 - h0)};
-                nbits = h1 > h0 ? col[h1 - 1] - (int32_t)r : 0;
+                k = chunks_of(class_of_order(ord), lv, work[r], pp);
             }
-#pragma unroll
-            for (int cc = 0; cc < TC_NUM_CLS; ++cc) {
-                const unsigned in = __ballot_sync(FULL, c == cc);
-                if (!in) continue;
-                const int64_t mine = c == cc ? k : 0;
-                ull o = base[cc];
-                if (__any_sync(FULL, mine > 1)) {
-                    ull incl = (ull)mine;
+            // place of this lane's first item in its order class; lane o keeps
+            // the running offset of order class o
+            ull at = 0;
+            for (unsigned todo = __ballot_sync(FULL, ord >= 0); todo;) {
+                const int o = __shfl_sync(FULL, ord, __ffs(todo) - 1);
+                const unsigned in = __ballot_sync(FULL, ord == o);
+                todo &= ~in;
+                const ull base = __shfl_sync(FULL, off, o);
+                ull incl = ord == o ? (ull)k : 0, total;
+                if (__any_sync(FULL, ord == o && k > 1)) {
+                    const ull mine = incl;
 #pragma unroll
                     for (int dd = 1; dd < 32; dd <<= 1) {
                         const ull y = __shfl_up_sync(FULL, incl, dd);
                         if (lane >= dd) incl += y;
                     }
-                    o += incl - (ull)mine;
-                    base[cc] += __shfl_sync(FULL, incl, 31);
+                    total = __shfl_sync(FULL, incl, 31);
+                    if (ord == o) at = base + incl - mine;
                 } else {
-                    o += (ull)__popc(in & below);
-                    base[cc] += (ull)__popc(in);
+                    total = (ull)__popc(in);
+                    if (ord == o) at = base + (ull)__popc(in & below);
                 }
-                if (c == cc)
-                    for (int64_t j = 0; j < mine; ++j) {
-                        tg.d[cc][o + j] = d;
-                        tg.nb[cc][o + j] = nbits;
-                        tg.pb[cc][o + j] = b + lv * j / k;
-                        tg.pe[cc][o + j] = b + lv * (j + 1) / k;
-                    }
+                if (lane == o) off += total;
+            }
+            if (ord >= 0) {
+                const int c = class_of_order(ord);
+                const tc_item d{h0, (int32_t)r, (int32_t)(h1 - h0)};
+                const int32_t nbits = h1 > h0 ? col[h1 - 1] - (int32_t)r : 0;
+                for (int64_t j = 0; j < k; ++j) {
+                    tg.d[c][at + j] = d;
+                    tg.nb[c][at + j] = nbits;
+                    tg.pb[c][at + j] = b + lv * j / k;
+                    tg.pe[c][at + j] = b + lv * (j + 1) / k;
+                }
             }
         }
     }
@@ -1413,7 +1443,7 @@ tc_status make_plan(tc_graph* g, int strategy, cudaStream_t s) {
     } while (0)
 #define PLAN_CUDA(x) PLAN_TRY(from_cuda(x))
     PLAN_TRY(dalloc((void**)&acc, sizeof(class_acc), s));
-    PLAN_TRY(dalloc((void**)&gsum, TC_NUM_CLS * (groups + 1) * 8, s));
+    PLAN_TRY(dalloc((void**)&gsum, kNumOrd * (groups + 1) * 8, s));
     PLAN_TRY(dalloc((void**)&cls, n + 1, s));
     PLAN_CUDA(cudaMemsetAsync(acc, 0, sizeof(class_acc), s));
     if (n > 0) {
@@ -1424,7 +1454,7 @@ tc_status make_plan(tc_graph* g, int strategy, cudaStream_t s) {
             PLAN_CUDA(cudaGetLastError());
         }
         launch_scope ls("plan_scan", s);
-        k_plan_scan<<<TC_NUM_CLS, kPlanScanThreads, 0, s>>>(gsum, groups);
+        k_plan_scan<<<kNumOrd, kPlanScanThreads, 0, s>>>(gsum, groups, gsum + kNumOrd * groups);
         PLAN_CUDA(cudaGetLastError());
     }
     class_acc h{};
@@ -1462,7 +1492,7 @@ tc_status make_plan(tc_graph* g, int strategy, cudaStream_t s) {
             tg.pe[c] = p.pe[c];
         }
         k_emit<<<blocks_for(groups * 32), 256, 0, s>>>(g->row_ptr, g->hstart, g->col, g->work, n, g->params, slices,
-                                                       groups, cls, gsum, tg);
+                                                       groups, cls, gsum, gsum + kNumOrd * groups, tg);
         PLAN_CUDA(cudaGetLastError());
     }
     // the bitmap kernels get the shared memory their largest item needs, not

@@ -69,8 +69,9 @@ __device__ __forceinline__ ull warp_sum(ull x) {
 // numer(r) = △(r) + Σ_{u ∈ N(r)} (u ∈ N△(r) ? 1 : 3)·△(u).  A tail entry
 // holds u in col and its flag in place; a head entry's record holds u and
 // the twin position where its flag sits.
-// Rows are in rank (= degree) order, so three contiguous rank bands get
-// one thread, one warp and one CTA per row.
+// Rows of degree up to 32, up to 4096 and above get one thread, one warp and
+// one CTA each: three contiguous rank bands of a single graph, lists of a
+// union's larger rows (`list`, with its other rows skipped by k_gather_thread).
 struct gather_args;
 __device__ __forceinline__ void finish_row(int64_t r, ull acc, const gather_args& a);
 
@@ -120,11 +121,11 @@ __device__ __forceinline__ void finish_row(int64_t r, ull acc, const gather_args
     if (a.tc_out) a.tc_out[v] = div_rn(acc, a.rank_graph ? a.den_graph[a.rank_graph[r]] : a.den);
 }
 
-// one thread per row, rows [r0, r1)
-__global__ void __launch_bounds__(256) k_gather_thread(gather_args a, int64_t r0, int64_t r1) {
-    for (int64_t r = r0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < r1;
-         r += (int64_t)gridDim.x * blockDim.x) {
+// one thread per row, rows [0, r1) of degree up to 32
+__global__ void __launch_bounds__(256) k_gather_thread(gather_args a, int64_t r1) {
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < r1; r += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = a.row_ptr[r], h = a.hstart[r], e = a.row_ptr[r + 1];
+        if (e - b > 32) continue;   // a union's mid or hub row
         ull acc = a.tri[r];
         for (int64_t p = b; p < h; ++p) acc += head_term(a, p);
         for (int64_t p = h; p < e; ++p) acc += tail_term(a, p);
@@ -132,11 +133,13 @@ __global__ void __launch_bounds__(256) k_gather_thread(gather_args a, int64_t r0
     }
 }
 
-// one warp per row, rows [r0, r1)
-__global__ void __launch_bounds__(256) k_gather_warp(gather_args a, int64_t r0, int64_t r1) {
+// one warp per row, `rows` rows from r0 on (or named by list)
+__global__ void __launch_bounds__(256)
+k_gather_warp(gather_args a, const int32_t* __restrict__ list, int64_t r0, int64_t rows) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t r = r0 + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5); r < r1; r += warps) {
+    for (int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; k < rows; k += warps) {
+        const int64_t r = list ? list[k] : r0 + k;
         const int64_t b = a.row_ptr[r], h = a.hstart[r], e = a.row_ptr[r + 1];
         ull acc = 0;
         for (int64_t p = b + lane; p < h; p += 32) acc += head_term(a, p);
@@ -146,11 +149,13 @@ __global__ void __launch_bounds__(256) k_gather_warp(gather_args a, int64_t r0, 
     }
 }
 
-// one CTA per row, rows [r0, r1)
-__global__ void __launch_bounds__(1024) k_gather_cta(gather_args a, int64_t r0, int64_t r1) {
+// one CTA per row, `rows` rows from r0 on (or named by list)
+__global__ void __launch_bounds__(1024)
+k_gather_cta(gather_args a, const int32_t* __restrict__ list, int64_t r0, int64_t rows) {
     __shared__ ull part[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t r = r0 + blockIdx.x; r < r1; r += gridDim.x) {
+    for (int64_t k = blockIdx.x; k < rows; k += gridDim.x) {
+        const int64_t r = list ? list[k] : r0 + k;
         const int64_t b = a.row_ptr[r], h = a.hstart[r], e = a.row_ptr[r + 1];
         ull acc = 0;
         for (int64_t p = b + threadIdx.x; p < h; p += blockDim.x) acc += head_term(a, p);
@@ -167,18 +172,33 @@ __global__ void __launch_bounds__(1024) k_gather_cta(gather_args a, int64_t r0, 
     }
 }
 
-// Σ_{v ∈ graph k} △(v) (= 3△(G_k)) for every graph of a batch; lanes of a
-// warp that hit the same graph add once.
+// Σ_{v ∈ graph k} △(v) (= 3△(G_k)) for every graph of a batch.  A union's
+// ranks keep a graph's vertices together, so each lane of a
+// warp that walks 32·kSumRounds consecutive ranks adds up in a register and
+// flushes when the graph changes.  (Matching lanes by graph and adding their
+// counts one by one took 1.28 ms on the 8192-graph batch.)
+constexpr int kSumRounds = 16;
 __global__ void k_graph_sums(const ull* __restrict__ tri, const int32_t* __restrict__ rank_graph, int64_t n,
                              ull* __restrict__ sums) {
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n;
-         r += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t k = rank_graph[r];
-        const ull t = tri[r];
-        const unsigned same = __match_any_sync(__activemask(), k);
-        ull sum = 0;
-        for (unsigned mm = same; mm; mm &= mm - 1) sum += __shfl_sync(same, t, __ffs(mm) - 1);
-        if ((threadIdx.x & 31) == __ffs(same) - 1 && sum) atomicAdd(&sums[k], sum);
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5), per = 32 * kSumRounds;
+    for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; c * per < n; c += warps) {
+        const int64_t r0 = c * per + (threadIdx.x & 31);
+        int32_t cur = -1;
+        ull acc = 0;
+#pragma unroll 4
+        for (int j = 0; j < kSumRounds; ++j) {
+            const int64_t r = r0 + 32 * j;
+            if (r >= n) break;
+            const int32_t k = rank_graph[r];
+            const ull t = tri[r];
+            if (k != cur) {
+                if (acc) atomicAdd(&sums[cur], acc);
+                acc = 0;
+                cur = k;
+            }
+            acc += t;
+        }
+        if (acc) atomicAdd(&sums[cur], acc);
     }
 }
 
@@ -252,21 +272,24 @@ tc_status run_centrality(tc_graph* g, uint64_t* d_numer, double* d_tc, cudaStrea
         k_tri32<<<blocks_for(n, 256), 256, 0, s>>>(g->tri, n, g->tri32);
         TC_LAUNCH_CHECK();
     }
-    const int64_t r1 = g->band[0], r2 = g->band[1];   // degree <= 32 | <= 4096 | larger
-    if (r1 > 0) {
+    // degree <= 32 | <= 4096 | larger
+    const int32_t* list = g->row_list;
+    const int64_t mids = list ? g->band[0] : g->band[1] - g->band[0], hubs = list ? g->band[1] : n - g->band[1];
+    const int64_t small = list ? n : g->band[0];
+    if (small > 0) {
         launch_scope ls("gather_thread", s);
-        k_gather_thread<<<blocks_for(r1, 256), 256, 0, s>>>(a, 0, r1);
+        k_gather_thread<<<blocks_for(small, 256), 256, 0, s>>>(a, small);
         TC_LAUNCH_CHECK();
     }
-    if (r2 > r1) {
+    if (mids > 0) {
         launch_scope ls("gather_warp", s);
-        k_gather_warp<<<blocks_for((r2 - r1) * 32, 256), 256, 0, s>>>(a, r1, r2);
+        k_gather_warp<<<blocks_for(mids * 32, 256), 256, 0, s>>>(a, list, g->band[0], mids);
         TC_LAUNCH_CHECK();
     }
-    if (n > r2) {
+    if (hubs > 0) {
         launch_scope ls("gather_cta", s);
-        const int64_t rows = n - r2;
-        k_gather_cta<<<(int)std::min<int64_t>(rows, (int64_t)sm_count() * 2), 1024, 0, s>>>(a, r2, n);
+        k_gather_cta<<<(int)std::min<int64_t>(hubs, (int64_t)sm_count() * 2), 1024, 0, s>>>(
+            a, list ? list + g->hub_at : nullptr, g->band[1], hubs);
         TC_LAUNCH_CHECK();
     }
     return TC_OK;
@@ -275,7 +298,7 @@ tc_status run_centrality(tc_graph* g, uint64_t* d_numer, double* d_tc, cudaStrea
 tc_status run_graph_sums(tc_graph* g, const int32_t* rank_graph, ull* sums, cudaStream_t s) {
     if (g->n == 0) return TC_OK;
     launch_scope ls("batch_graph_sums", s);
-    k_graph_sums<<<blocks_for(g->n, 256), 256, 0, s>>>(g->tri, rank_graph, g->n, sums);
+    k_graph_sums<<<blocks_for((g->n + kSumRounds - 1) / kSumRounds, 256), 256, 0, s>>>(g->tri, rank_graph, g->n, sums);
     TC_LAUNCH_CHECK();
     return TC_OK;
 }

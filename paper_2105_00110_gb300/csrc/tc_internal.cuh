@@ -108,7 +108,13 @@ struct tc_graph {
     tc_head* head = nullptr;
     int64_t* edge_tail = nullptr;
     int64_t* work = nullptr;             // [n] W(v) = Σ_{u ∈ N_L(v)} hrem(u, v)
-    int64_t band[2] = {0, 0};            // first rank of degree > 32, of degree > 4096
+    // rows by degree: up to 32, up to 4096 (mid), above (hub).  A single graph's
+    // degrees ascend with rank: band holds the first mid and the first hub
+    // rank.  A union keeps each graph's ranks together: band holds how many
+    // mid and hub rows there are and row_list names them, hubs from hub_at.
+    int64_t band[2] = {0, 0};
+    int32_t* row_list = nullptr;
+    int64_t hub_at = 0;
     tc_plan plan;
     // workspace of tc_count / tc_centrality
     unsigned long long* tri = nullptr;   // [n], rank space
@@ -297,9 +303,18 @@ cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, size_t smem, c
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
-// build pieces (tc_build.cu)
+// build pieces (tc_build.cu).  A union of many graphs is built from the
+// graphs' own pairs and labels: graph k has the pairs [poff[k], poff[k+1])
+// with ids in [0, voff[k+1] - voff[k]), its labels start at voff[k].
+struct union_layout {
+    const int64_t* poff;     // [G+1] device
+    const int64_t* voff;     // [G+1] device
+    int64_t G;
+    int64_t max_n;           // vertices of the largest graph
+    int32_t* rank_graph;     // [n] device, receives the graph of every rank
+};
 tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np, int64_t n,
-                      uint32_t flags, cudaStream_t s);
+                      uint32_t flags, cudaStream_t s, const union_layout* un = nullptr);
 void free_graph_memory(tc_graph* g);
 
 // dense core (tc_core.cu).  Build flag for unions of many graphs, which
