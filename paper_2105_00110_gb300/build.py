@@ -22,7 +22,7 @@ BUILD_INFO = os.path.join(BUILD, "build_info.json")
 # the bounds-checked variant (-DTC_DEBUG_BOUNDS), built on request for tests
 DEBUG_BUILD = os.path.join(HERE, "_build_debug")
 DEBUG_LIB = os.path.join(DEBUG_BUILD, "libtc_gb300.so")
-SOURCES = ["tc_api.cu", "tc_build.cu", "tc_count.cu", "tc_core.cu", "tc_gather.cu", "tc_batch.cu", "tc_noalloc.cu",
+SOURCES = ["tc_api.cu", "tc_build.cu", "tc_sort.cu", "tc_count.cu", "tc_core.cu", "tc_gather.cu", "tc_batch.cu", "tc_noalloc.cu",
            "tc_server.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INCLUDE, "-I" + CSRC]

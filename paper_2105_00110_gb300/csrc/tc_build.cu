@@ -30,6 +30,7 @@ namespace tcx {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int64_t kMsdPairs = 1 << 19;            // pairs from which the keys are sorted by tc_sort.cu
 constexpr int64_t kMaxDegreeReadBack = 1 << 20;   // vertices above which the largest degree is read back
 
 inline int grid_for(int64_t n, int per_thread = 1) {
@@ -42,10 +43,35 @@ inline int grid_for(int64_t n, int per_thread = 1) {
 #define GRID_STRIDE(i, n) \
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (n); i += (int64_t)gridDim.x * blockDim.x)
 
+// Pairs -> canonical keys (lower label, higher label), ~0 for a self-loop or
+// a bad id.  With cnt, also how many keys have each value of their top
+// bits (key >> shift, `bins` of them): the first digit of the sort.
+struct digit_counts {
+    uint32_t* cnt;   // null: not wanted
+    int shift, bins;
+};
+constexpr int kMaxFirstBins = 1024;
+__device__ __forceinline__ void digit_add(const digit_counts& dc, uint32_t* h, uint64_t key) {
+    if (dc.cnt && key != ~0ull) atomicAdd(&h[key >> dc.shift], 1u);
+}
+__device__ __forceinline__ void digit_begin(const digit_counts& dc, uint32_t* h) {
+    if (!dc.cnt) return;
+    for (int b = threadIdx.x; b < dc.bins; b += blockDim.x) h[b] = 0;
+    __syncthreads();
+}
+__device__ __forceinline__ void digit_end(const digit_counts& dc, uint32_t* h) {
+    if (!dc.cnt) return;
+    __syncthreads();
+    for (int b = threadIdx.x; b < dc.bins; b += blockDim.x)
+        if (h[b]) atomicAdd(&dc.cnt[b], h[b]);
+}
+
 template <typename T>
 __global__ void k_make_keys(const T* __restrict__ src, const T* __restrict__ dst, int64_t np,
                             int64_t n, int bits, uint64_t* __restrict__ keys,
-                            unsigned int* __restrict__ err) {
+                            unsigned int* __restrict__ err, digit_counts dc) {
+    __shared__ uint32_t h[kMaxFirstBins];
+    digit_begin(dc, h);
     GRID_STRIDE(i, np) {
         int64_t a = (int64_t)src[i], b = (int64_t)dst[i];
         uint64_t key = ~0ull;
@@ -56,7 +82,9 @@ __global__ void k_make_keys(const T* __restrict__ src, const T* __restrict__ dst
             key = (lo << bits) | hi;
         }
         keys[i] = key;
+        digit_add(dc, h, key);
     }
+    digit_end(dc, h);
 }
 
 // The same for a union's pairs (ids local to their graph): a warp takes
@@ -68,7 +96,10 @@ __global__ void k_make_keys(const T* __restrict__ src, const T* __restrict__ dst
 constexpr int kUnionChunk = 32 * 32;
 template <typename T>
 __global__ void k_make_union_keys(const T* __restrict__ src, const T* __restrict__ dst, int64_t np, union_layout un,
-                                  int dbits, uint64_t* __restrict__ keys, unsigned int* __restrict__ err) {
+                                  int dbits, uint64_t* __restrict__ keys, unsigned int* __restrict__ err,
+                                  digit_counts dc) {
+    __shared__ uint32_t h[kMaxFirstBins];
+    digit_begin(dc, h);
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int64_t chunks = (np + kUnionChunk - 1) / kUnionChunk;
@@ -96,8 +127,10 @@ __global__ void k_make_union_keys(const T* __restrict__ src, const T* __restrict
             else if (a < b) key = ((uint64_t)(v0 + a) << dbits) | (uint64_t)(b - a);
             else if (b < a) key = ((uint64_t)(v0 + b) << dbits) | (uint64_t)(a - b);
             keys[i] = key;
+            digit_add(dc, h, key);
         }
     }
+    digit_end(dc, h);
     if (bad) atomicOr(err, 1u);
 }
 
@@ -1009,47 +1042,65 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
     if (np > 0) {
         TC_TRY(sc.get(&ka, np));
         TC_TRY(sc.get(&kb, np));
+        const int key_bits = bits + low_bits;
+        const bool msd = np >= kMsdPairs && np < ((int64_t)1 << 32);   // 32-bit counts in the sort
+        digit_counts dc{};
+        if (msd) {
+            const int d0 = sort_first_digit(np, key_bits);
+            dc.bins = 1 << d0;
+            dc.shift = key_bits - d0;
+            TC_TRY(sc.get(&dc.cnt, dc.bins));
+            TC_CUDA(cudaMemsetAsync(dc.cnt, 0, dc.bins * 4, s));
+        }
         {
             launch_scope ls("build_make_keys", s);
             if (un && i32)
                 k_make_union_keys<int32_t><<<grid_for(np, 8), kThreads, 0, s>>>(
-                    (const int32_t*)dsrc, (const int32_t*)ddst, np, *un, low_bits, ka, err);
+                    (const int32_t*)dsrc, (const int32_t*)ddst, np, *un, low_bits, ka, err, dc);
             else if (un)
                 k_make_union_keys<int64_t><<<grid_for(np, 8), kThreads, 0, s>>>(
-                    (const int64_t*)dsrc, (const int64_t*)ddst, np, *un, low_bits, ka, err);
+                    (const int64_t*)dsrc, (const int64_t*)ddst, np, *un, low_bits, ka, err, dc);
             else if (i32)
                 k_make_keys<int32_t><<<grid_for(np), kThreads, 0, s>>>(
-                    (const int32_t*)dsrc, (const int32_t*)ddst, np, n, bits, ka, err);
+                    (const int32_t*)dsrc, (const int32_t*)ddst, np, n, bits, ka, err, dc);
             else
                 k_make_keys<int64_t><<<grid_for(np), kThreads, 0, s>>>(
-                    (const int64_t*)dsrc, (const int64_t*)ddst, np, n, bits, ka, err);
+                    (const int64_t*)dsrc, (const int64_t*)ddst, np, n, bits, ka, err, dc);
             TC_LAUNCH_CHECK();
         }
-        cub::DoubleBuffer<uint64_t> kbuf(ka, kb);
-        {
+        uint64_t *sorted = nullptr, *uniq = nullptr;
+        int64_t count = np;
+        if (msd) {
+            TC_TRY(sort_keys_msd([&](void** q, size_t bytes) { return sc.get((uint8_t**)q, bytes); }, ka, kb, dc.cnt,
+                                 np, key_bits, err, &sorted, &count, s));
+            uniq = sorted == ka ? kb : ka;
+        } else {
+            cub::DoubleBuffer<uint64_t> kbuf(ka, kb);
             launch_scope ls("build_sort_pairs", s);
-            TC_TRY(sort_keys(sc, kbuf, np, bits + low_bits, s));
-        }
-        uint64_t* sorted = kbuf.Current();
-        uint64_t* uniq = kbuf.Alternate();
-        size_t bytes = 0;
-        TC_CUDA(cub::DeviceSelect::Unique(nullptr, bytes, sorted, uniq, d_nsel, np, s));
-        uint8_t* tmp = nullptr;
-        TC_TRY(sc.get(&tmp, bytes));
-        {
-            launch_scope ls("build_unique", s);
-            TC_TRY(run_library("select_unique", np, 0, true, s, [&](cudaStream_t st) {
-                return cub::DeviceSelect::Unique(tmp, bytes, sorted, uniq, d_nsel, np, st);
-            }));
+            TC_TRY(sort_keys(sc, kbuf, np, key_bits, s));
+            sorted = kbuf.Current();
+            uniq = kbuf.Alternate();
         }
         int64_t h_sel = 0;
         uint64_t last = 0;
         unsigned int h_err = 0;
-        TC_CUDA(cudaMemcpyAsync(&h_sel, d_nsel, 8, cudaMemcpyDeviceToHost, s));
-        TC_CUDA(cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, s));
-        TC_CUDA(cudaStreamSynchronize(s));
-        if (h_err) return TC_ERR_INVALID_ARG;
-        if (h_sel > 0) {
+        if (count > 0) {
+            size_t bytes = 0;
+            TC_CUDA(cub::DeviceSelect::Unique(nullptr, bytes, sorted, uniq, d_nsel, count, s));
+            uint8_t* tmp = nullptr;
+            TC_TRY(sc.get(&tmp, bytes));
+            {
+                launch_scope ls("build_unique", s);
+                TC_TRY(run_library("select_unique", np, 0, true, s, [&](cudaStream_t st) {
+                    return cub::DeviceSelect::Unique(tmp, bytes, sorted, uniq, d_nsel, count, st);
+                }));
+            }
+            TC_CUDA(cudaMemcpyAsync(&h_sel, d_nsel, 8, cudaMemcpyDeviceToHost, s));
+            TC_CUDA(cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, s));
+            TC_CUDA(cudaStreamSynchronize(s));
+            if (h_err) return TC_ERR_INVALID_ARG;
+        }
+        if (h_sel > 0 && !msd) {   // loops sort last, as one key of all ones
             TC_CUDA(cudaMemcpyAsync(&last, uniq + h_sel - 1, 8, cudaMemcpyDeviceToHost, s));
             TC_CUDA(cudaStreamSynchronize(s));
         }

@@ -317,6 +317,17 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
                       uint32_t flags, cudaStream_t s, const union_layout* un = nullptr);
 void free_graph_memory(tc_graph* g);
 
+// sort of the canonical keys from the most significant digit (tc_sort.cu).
+// `keys` (np of them, `bits` significant; ~0: dropped) and `other` are its two
+// buffers; first_counts holds how many keys have each value of their first
+// digit, the top sort_first_digit(np, bits) bits.  *sorted receives the buffer
+// with the *valid sorted keys.  Temporaries come from `get`.  Synchronises s;
+// TC_ERR_INVALID_ARG if the error word *err (device) is set by then.
+typedef std::function<tc_status(void**, size_t)> sort_alloc;
+int sort_first_digit(int64_t np, int bits);
+tc_status sort_keys_msd(const sort_alloc& get, uint64_t* keys, uint64_t* other, uint32_t* first_counts, int64_t np,
+                        int bits, const unsigned int* err, uint64_t** sorted, int64_t* valid, cudaStream_t s);
+
 // dense core (tc_core.cu).  Build flag for unions of many graphs, which
 // have no dense core: the build never sets one up.
 constexpr uint32_t TC_BUILD_NO_CORE = 1u << 30;

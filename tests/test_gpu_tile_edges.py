@@ -113,3 +113,54 @@ def wheels(*rims):
                          ids=lambda r: "-".join(map(str, r)))
 def test_hub_rows(rims):
     check_full(*wheels(*rims))
+
+
+def sort_inputs(kind, p):
+    rng = np.random.default_rng(p)
+    if kind == "uniform":                 # buckets of like size
+        n = 1 << 21
+        return rng.integers(0, n, p), rng.integers(0, n, p), n
+    if kind == "one-pair":                # one key, p times: bits run out
+        return np.full(p, 7), np.full(p, 3), 1 << 20
+    if kind == "few-keys":                # a small key space, every key many times
+        return rng.integers(0, 40, p), rng.integers(0, 40, p), 40
+    if kind == "loops":                   # nothing left
+        a = rng.integers(0, 1000, p)
+        return a, a, 1000
+    if kind == "star":                    # one row holds everything, in order
+        return np.zeros(p, np.int64), np.arange(1, p + 1), p + 1
+    if kind == "hubs":                    # rows of several sizes beside light ones
+        n = 1 << 20
+        hub = rng.choice([5, 6, 70000, 70001, n - 2], p)
+        return np.where(rng.random(p) < 0.6, hub, rng.integers(0, n, p)), rng.integers(0, n, p), n
+    if kind == "clustered":               # higher ends crowd together: crowded sub-bins
+        n = 1 << 22
+        a = rng.integers(0, 64, p)
+        return a, 1000 + (np.abs(rng.normal(0, 40, p))).astype(np.int64), n
+    n = 3_000_001                         # ragged: n above a power of two, wide keys
+    return (rng.random(p) ** 3 * n).astype(np.int64), rng.integers(0, n, p), n
+
+
+@pytest.mark.parametrize("ids", [np.int32, np.int64])
+@pytest.mark.parametrize("kind,p", [("uniform", 1 << 19), ("uniform", (1 << 20) + 1), ("one-pair", 600_000),
+                                    ("few-keys", 700_001), ("loops", 1 << 19), ("star", (1 << 20) - 1),
+                                    ("hubs", 3_000_000), ("clustered", 1 << 20), ("ragged", 2_500_003),
+                                    ("uniform", (1 << 19) - 1)])
+def test_sorted_edges(kind, p, ids):
+    src, dst, n = sort_inputs(kind, p)
+    g = tcg.Graph(torch.from_numpy(src.astype(ids)).cuda(), torch.from_numpy(dst.astype(ids)).cuda(), n)
+    lo, hi = np.minimum(src, dst).astype(np.int64), np.maximum(src, dst).astype(np.int64)
+    key = np.unique((lo * n + hi)[lo != hi])
+    u, v = (x.cpu().numpy() for x in g.edges())
+    assert g.m == len(key) and np.array_equal(u, key // n) and np.array_equal(v, key % n)
+    g.close()
+
+
+def test_sort_rejects_a_bad_id():
+    src = np.arange(1 << 19, dtype=np.int32) % 1000
+    for at, bad in ((12345, 1000), ((1 << 19) - 1, -1)):
+        dst = np.roll(src, 1)
+        dst[at] = bad
+        with pytest.raises(tcg.TCError) as e:
+            tcg.Graph(torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), 1000)
+        assert e.value.status == tcg.TC_ERR_INVALID_ARG
