@@ -888,7 +888,10 @@ k_count_cta(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col
             if (MERGE) {
                 merge_streams<T, EC>(lane, (NC * warp) / (T / 32), (NC * (warp + 1)) / (T / 32), tb, ls.ids, hv, cnt, col, flag, dm);
             } else {
-                const int gb = (int)(((int64_t)GT * warp) / (T / 32)), ge = (int)(((int64_t)GT * (warp + 1)) / (T / 32));
+                // whole windows of 32 groups to the warps: only the round's last
+                // window can be partly empty, not one of every warp
+                const int NW = (GT + 31) >> 5;
+                const int gb = 32 * ((NW * warp) / (T / 32)), ge = min(GT, 32 * ((NW * (warp + 1)) / (T / 32)));
                 if (LOOK == L_BITMAP)
                     walk_groups<lookup_bitmap, true, T, kCtaG, EC>(lane, tb, NC, gb, ge, lb, cnt, h0, col, tri, flag, dm);
                 else if (LOOK == L_SORTED)
