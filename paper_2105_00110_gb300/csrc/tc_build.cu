@@ -40,6 +40,13 @@ inline int grid_for(int64_t n, int per_thread = 1) {
     return (int)std::min(want, cap);
 }
 
+// One chunk of `chunk` items a block, however many blocks: blocks start in
+// order, so the items in work at a time are neighbours and what they scatter
+// to nearby places meets in L2.  (A grid of 16 CTAs an SM striding over all
+// items sweeps them two to three times, each sweep touching every place: the
+// 8192-graph batch's edges took 12.4 ms to scatter that way, 7.3 in order.)
+inline int ordered_blocks(int64_t n, int64_t chunk) { return (int)std::max<int64_t>(1, (n + chunk - 1) / chunk); }
+
 #define GRID_STRIDE(i, n) \
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (n); i += (int64_t)gridDim.x * blockDim.x)
 
@@ -282,17 +289,26 @@ __global__ void k_hstart(const int64_t* __restrict__ row_ptr, const int32_t* __r
 
 // Each edge to the next free slot of its lower end's run (row r's run
 // starts at hptr[r]) as (hi << 32) | edge id, so that sorting each run puts
-// N_H(lo) in order with the edge ids alongside.
+// N_H(lo) in order with the edge ids alongside.  A block takes
+// kThreads * kPlace consecutive edges, kPlace cursor atomics a thread in flight.
+constexpr int kPlace = 4;
 template <class C>
-__global__ void k_tail_place(const uint64_t* __restrict__ keys, int64_t m, int bits, C* __restrict__ tnext,
-                             uint64_t* __restrict__ slot) {
+__global__ void __launch_bounds__(kThreads)
+k_tail_place(const uint64_t* __restrict__ keys, int64_t m, int bits, C* __restrict__ tnext,
+             uint64_t* __restrict__ slot) {
     const uint64_t mask = (1ull << bits) - 1;
-    GRID_STRIDE(e, m) {
-        const uint64_t k = keys[e];
-        const uint64_t lo = k >> bits, hi = k & mask;
-        const int64_t i = (int64_t)atomicAdd(&tnext[lo], (C)1);
-        slot[i] = (hi << 32) | (uint64_t)e;
-    }
+    const int64_t e0 = blockIdx.x * (int64_t)(kThreads * kPlace) + threadIdx.x;
+    uint64_t k[kPlace];
+    int64_t at[kPlace];
+#pragma unroll
+    for (int j = 0; j < kPlace; ++j)
+        if (e0 + j * kThreads < m) k[j] = keys[e0 + j * kThreads];
+#pragma unroll
+    for (int j = 0; j < kPlace; ++j)
+        if (e0 + j * kThreads < m) at[j] = (int64_t)atomicAdd(&tnext[k[j] >> bits], (C)1);
+#pragma unroll
+    for (int j = 0; j < kPlace; ++j)
+        if (e0 + j * kThreads < m) slot[at[j]] = ((k[j] & mask) << 32) | (uint64_t)(e0 + j * kThreads);
 }
 
 // Both entries of one edge, from the i-th element x of row r's sorted run
@@ -300,11 +316,12 @@ __global__ void k_tail_place(const uint64_t* __restrict__ keys, int64_t m, int b
 // canonical id -> t, and the head entry in row hi (N_L(hi) in any order) at
 // the next free slot of its cursor, as the record
 // {r, |{w ∈ N_H(r) : w > hi}| = e - t - 1, twin = t}.
+template <class C>
 __device__ __forceinline__ void write_tail(int64_t r, int64_t t, int64_t e, uint64_t x, int64_t hp,
                                            int32_t* __restrict__ col, tc_head* __restrict__ head,
-                                           int64_t* __restrict__ edge_tail, int64_t core_t) {
+                                           C* __restrict__ edge_tail, int64_t core_t) {
     col[t] = (int32_t)(x >> 32);
-    edge_tail[x & 0xffffffffull] = t;
+    edge_tail[x & 0xffffffffull] = (C)t;
     tc_head rec;
     rec.u = (int32_t)r;
     // a lower end in the dense core (ranks >= core_t) streams nothing: the
@@ -317,7 +334,7 @@ __device__ __forceinline__ void write_tail(int64_t r, int64_t t, int64_t e, uint
 template <class C>
 __device__ __forceinline__ void emit_tail(int64_t r, int64_t t, int64_t e, uint64_t x, C* __restrict__ hnext,
                                           int32_t* __restrict__ col, tc_head* __restrict__ head,
-                                          int64_t* __restrict__ edge_tail, int64_t core_t) {
+                                          C* __restrict__ edge_tail, int64_t core_t) {
     const int64_t hp = (int64_t)atomicAdd(&hnext[(int32_t)(x >> 32)], (C)1);
     write_tail(r, t, e, x, hp, col, head, edge_tail, core_t);
 }
@@ -369,7 +386,8 @@ constexpr int kMidShort = TC_MID_SHORT;   // longest run of the one-warp tier (5
 // and stores a lane are in flight together.  Bound by the latency of those
 // scattered stores and by issue; a network over the warp's registers, eight
 // runs at a time with a run in the first lanes of each register, kept 3 of 32
-// lanes busy on the 8192-graph batch (4096^2 grid: 6.4 -> 5.6 ms).
+// lanes busy on the 8192-graph batch (4096^2 grid: 6.4 -> 5.6 ms; with the
+// blocks in order 4.5, and 12.3 -> 7.1 on the batch).
 // Longer runs are queued: 33..kMidShort tails from the front of `big`
 // (count nbig[0]) and kMidShort+1..kMidRun tails from the back of its first
 // n entries (count nbig[1]) for k_runs_mid, which never meet since there are
@@ -389,7 +407,7 @@ __global__ void __launch_bounds__(kThreads)
 k_runs_small(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart,
              const int64_t* __restrict__ hptr, const uint64_t* __restrict__ slot, int64_t n,
              C* __restrict__ hnext, int32_t* __restrict__ col, tc_head* __restrict__ head,
-             int64_t* __restrict__ edge_tail, int32_t* __restrict__ big,
+             C* __restrict__ edge_tail, int32_t* __restrict__ big,
              unsigned int* __restrict__ nbig, int64_t core_t) {
     __shared__ small_runs s_runs[kThreads / 32];
     small_runs& sr = s_runs[threadIdx.x >> 5];
@@ -475,7 +493,7 @@ __global__ void __launch_bounds__(32 * kMidWarps)
 k_runs_mid(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart,
            const int64_t* __restrict__ hptr, const uint64_t* __restrict__ slot, const int32_t* __restrict__ big,
            const unsigned int* __restrict__ nbig, int64_t n, C* __restrict__ hnext, int32_t* __restrict__ col,
-           tc_head* __restrict__ head, int64_t* __restrict__ edge_tail, int64_t core_t) {
+           tc_head* __restrict__ head, C* __restrict__ edge_tail, int64_t core_t) {
     static_assert(CAP == kMidShort || CAP == kMidRun, "one queue per capacity");
     static_assert(kMidShort == 256 || kMidShort == 512, "register sort tiers: up to 16 keys a lane");
     constexpr bool kBack = CAP == kMidRun;
@@ -564,7 +582,7 @@ __device__ __forceinline__ void sort_run_regs(uint64_t (&x)[E], int lane) {
 template <class C, int E>
 __device__ __forceinline__ void run_regs(int lane, int64_t r, int64_t i0, int len, const uint64_t* __restrict__ slot,
                                          int64_t h, int64_t end, C* __restrict__ hnext, int32_t* __restrict__ col,
-                                         tc_head* __restrict__ head, int64_t* __restrict__ edge_tail, int64_t core_t) {
+                                         tc_head* __restrict__ head, C* __restrict__ edge_tail, int64_t core_t) {
     uint64_t x[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
@@ -584,7 +602,7 @@ __global__ void __launch_bounds__(32 * kMidWarps)
 k_runs_mid_reg(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart,
                const int64_t* __restrict__ hptr, const uint64_t* __restrict__ slot, const int32_t* __restrict__ big,
                const unsigned int* __restrict__ nbig, C* __restrict__ hnext, int32_t* __restrict__ col,
-               tc_head* __restrict__ head, int64_t* __restrict__ edge_tail, int64_t core_t) {
+               tc_head* __restrict__ head, C* __restrict__ edge_tail, int64_t core_t) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned count = nbig[0];
     const unsigned warps = gridDim.x * kMidWarps;
@@ -685,7 +703,7 @@ template <class C, int E>
 __device__ __forceinline__ void run_cta(int lane, int w, uint64_t* sx, int64_t r, int64_t i0, int len,
                                         const uint64_t* __restrict__ slot, int64_t h, int64_t end,
                                         C* __restrict__ hnext, int32_t* __restrict__ col,
-                                        tc_head* __restrict__ head, int64_t* __restrict__ edge_tail, int64_t core_t) {
+                                        tc_head* __restrict__ head, C* __restrict__ edge_tail, int64_t core_t) {
     uint64_t x[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
@@ -705,7 +723,7 @@ __global__ void __launch_bounds__(32 * kMidWarps)
 k_runs_long_cta(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart,
                 const int64_t* __restrict__ hptr, const uint64_t* __restrict__ slot, const int32_t* __restrict__ big,
                 const unsigned int* __restrict__ nbig, int64_t n, C* __restrict__ hnext, int32_t* __restrict__ col,
-                tc_head* __restrict__ head, int64_t* __restrict__ edge_tail, int64_t core_t) {
+                tc_head* __restrict__ head, C* __restrict__ edge_tail, int64_t core_t) {
     static_assert(32 * 8 * kMidWarps == kMidRun, "eight keys a thread cover the longest queued run");
     __shared__ uint64_t sx[kMidRun];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -731,7 +749,7 @@ __global__ void __launch_bounds__(kRunThreads)
 k_runs_big(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart,
            const int64_t* __restrict__ hptr, uint64_t* __restrict__ slot, const int32_t* __restrict__ big,
            const unsigned int* __restrict__ nbig, int64_t n, C* __restrict__ hnext, int32_t* __restrict__ col,
-           tc_head* __restrict__ head, int64_t* __restrict__ edge_tail, int64_t core_t) {
+           tc_head* __restrict__ head, C* __restrict__ edge_tail, int64_t core_t) {
     __shared__ uint64_t sk[kRunSmem];
     const unsigned count = nbig[2];
     for (unsigned q = blockIdx.x; q < count; q += gridDim.x) {
@@ -950,7 +968,7 @@ tc_status sort_by_key(scratch& sc, cub::DoubleBuffer<uint32_t>& keys, cub::Doubl
 template <class C>
 tc_status build_runs(tc_graph* g, cudaStream_t s, int64_t m, int64_t n, int bits, const uint64_t* keys,
                      uint64_t* slot, const int32_t* dh, const int64_t* hptr, int32_t* big, unsigned int* nbig,
-                     C* hnext, C* tnext, int rows_blocks, int64_t core_t) {
+                     C* hnext, C* tnext, int64_t core_t) {
     {
         launch_scope ls("build_hstart", s);
         k_hstart<<<grid_for(n), kThreads, 0, s>>>(g->row_ptr, dh, hptr, n, g->hstart, hnext, tnext, g->work);
@@ -958,39 +976,39 @@ tc_status build_runs(tc_graph* g, cudaStream_t s, int64_t m, int64_t n, int bits
     }
     {
         launch_scope ls("build_tail_place", s);
-        k_tail_place<<<grid_for(m), kThreads, 0, s>>>(keys, m, bits, tnext, slot);
+        k_tail_place<<<ordered_blocks(m, kThreads * kPlace), kThreads, 0, s>>>(keys, m, bits, tnext, slot);
         TC_LAUNCH_CHECK();
     }
     {
         launch_scope ls("build_runs_small", s);
-        k_runs_small<<<rows_blocks, kThreads, 0, s>>>(g->row_ptr, g->hstart, hptr, slot, n, hnext, g->col,
-                                                      g->head, g->edge_tail, big, nbig, core_t);
+        k_runs_small<<<ordered_blocks(n, kThreads), kThreads, 0, s>>>(g->row_ptr, g->hstart, hptr, slot, n, hnext, g->col,
+                                                      g->head, (C*)g->edge_tail, big, nbig, core_t);
         TC_LAUNCH_CHECK();
     }
     {
         launch_scope ls("build_runs_mid", s);
         if (TC_RUNS_REG)
             k_runs_mid_reg<C><<<sm_count() * 16, 32 * kMidWarps, 0, s>>>(
-                g->row_ptr, g->hstart, hptr, slot, big, nbig, hnext, g->col, g->head, g->edge_tail, core_t);
+                g->row_ptr, g->hstart, hptr, slot, big, nbig, hnext, g->col, g->head, (C*)g->edge_tail, core_t);
         else
             k_runs_mid<C, kMidShort><<<sm_count() * 16, 32 * kMidWarps, 0, s>>>(
-                g->row_ptr, g->hstart, hptr, slot, big, nbig, n, hnext, g->col, g->head, g->edge_tail, core_t);
+                g->row_ptr, g->hstart, hptr, slot, big, nbig, n, hnext, g->col, g->head, (C*)g->edge_tail, core_t);
         TC_LAUNCH_CHECK();
     }
     {
         launch_scope ls("build_runs_long", s);
         if (TC_RUNS_CTA_REG)
             k_runs_long_cta<C><<<sm_count() * 16, 32 * kMidWarps, 0, s>>>(
-                g->row_ptr, g->hstart, hptr, slot, big, nbig, n, hnext, g->col, g->head, g->edge_tail, core_t);
+                g->row_ptr, g->hstart, hptr, slot, big, nbig, n, hnext, g->col, g->head, (C*)g->edge_tail, core_t);
         else
             k_runs_mid<C, kMidRun><<<sm_count() * 8, 32 * kMidWarps, 0, s>>>(
-                g->row_ptr, g->hstart, hptr, slot, big, nbig, n, hnext, g->col, g->head, g->edge_tail, core_t);
+                g->row_ptr, g->hstart, hptr, slot, big, nbig, n, hnext, g->col, g->head, (C*)g->edge_tail, core_t);
         TC_LAUNCH_CHECK();
     }
     {
         launch_scope ls("build_runs_big", s);
         k_runs_big<<<sm_count() * 2, kRunThreads, 0, s>>>(g->row_ptr, g->hstart, hptr, slot, big, nbig, n,
-                                                          hnext, g->col, g->head, g->edge_tail, core_t);
+                                                          hnext, g->col, g->head, (C*)g->edge_tail, core_t);
         TC_LAUNCH_CHECK();
     }
     return TC_OK;
@@ -1122,7 +1140,7 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
     TC_CUDA(cudaMemsetAsync(g->col + e2, 0xff, 32 * 4, s));
     TC_TRY(dalloc((void**)&g->hstart, (n + 1) * 8, s));
     TC_TRY(dalloc((void**)&g->head, (e2 + 1) * sizeof(tc_head), s));
-    TC_TRY(dalloc((void**)&g->edge_tail, (m + 1) * 8, s));
+    TC_TRY(dalloc(&g->edge_tail, (m + 1) * (g->narrow() ? 4 : 8), s));
     TC_TRY(dalloc((void**)&g->work, (n + 1) * 8, s));
     TC_TRY(dalloc((void**)&g->tri, (n + 1) * 8, s));
     TC_TRY(dalloc((void**)&g->tri32, (n + 1) * 4, s));
@@ -1135,7 +1153,7 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
     TC_CUDA(cudaMemsetAsync(deg, 0, (n + 1) * 4, s));
     if (m > 0) {
         launch_scope ls("build_edges_degrees", s);
-        k_edges_degrees<<<grid_for(m), kThreads, 0, s>>>(ka, m, low_bits, un != nullptr, g->edge_u, g->edge_v,
+        k_edges_degrees<<<ordered_blocks(m, kThreads), kThreads, 0, s>>>(ka, m, low_bits, un != nullptr, g->edge_u, g->edge_v,
                                                          deg);
         TC_LAUNCH_CHECK();
     }
@@ -1198,7 +1216,7 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
             TC_TRY(sort_by_key(sc, rbuf, lbuf, n, rk.dbits + rk.gbits, s));
         }
         launch_scope ls("build_rank_apply", s);
-        k_rank_apply<<<grid_for(n), kThreads, 0, s>>>(rbuf.Current(), lbuf.Current(), n, rk.dbits, lg, g->perm, rank,
+        k_rank_apply<<<ordered_blocks(n, kThreads), kThreads, 0, s>>>(rbuf.Current(), lbuf.Current(), n, rk.dbits, lg, g->perm, rank,
                                                       degr, un ? un->rank_graph : nullptr, d_band, g->row_list,
                                                       g->hub_at);
         TC_LAUNCH_CHECK();
@@ -1227,20 +1245,22 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
         void* hnext = nullptr;   // head cursors (absolute positions)
         void* tnext = nullptr;   // tail-run cursors (compact order)
         int64_t* hptr = nullptr;
-        const bool narrow = e2 < ((int64_t)1 << 32);   // 32-bit cursors suffice
         TC_TRY(sc.get(&keys, m));
         TC_TRY(sc.get(&slot, m));
         TC_TRY(sc.get(&dh, n + 1));
         TC_TRY(sc.get(&big, n + m / kMidRun + 2));
         TC_TRY(sc.get(&nbig, 3));
-        TC_TRY(sc.get((uint8_t**)&hnext, (n + 1) * (narrow ? 4 : 8)));
-        TC_TRY(sc.get((uint8_t**)&tnext, (n + 1) * (narrow ? 4 : 8)));
+        TC_TRY(sc.get((uint8_t**)&hnext, (n + 1) * (g->narrow() ? 4 : 8)));
+        TC_TRY(sc.get((uint8_t**)&tnext, (n + 1) * (g->narrow() ? 4 : 8)));
         TC_TRY(sc.get(&hptr, n + 1));
         TC_CUDA(cudaMemsetAsync(dh, 0, (n + 1) * 4, s));
         TC_CUDA(cudaMemsetAsync(nbig, 0, 3 * sizeof(unsigned int), s));
         {
+            // in order where a graph's ranks are neighbours (the 8192-graph batch:
+            // 2.45 -> 1.78 ms); in a single graph neighbouring edges then add to
+            // the same few counters at once (R-MAT scale 24: 2.6 -> 4.1)
             launch_scope ls("build_edge_rank_keys", s);
-            k_edge_rank_keys<<<grid_for(m), kThreads, 0, s>>>(g->edge_u, g->edge_v, rank, m, bits, keys, dh);
+            k_edge_rank_keys<<<un ? ordered_blocks(m, kThreads) : grid_for(m), kThreads, 0, s>>>(g->edge_u, g->edge_v, rank, m, bits, keys, dh);
             TC_LAUNCH_CHECK();
         }
         size_t sbytes = 0;
@@ -1253,17 +1273,15 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
                 return cub::DeviceScan::ExclusiveSum(tmp, sbytes, dh, hptr, n + 1, st);
             }));
         }
-        const int cap = sm_count() * 16;
-        const int rows_blocks = (int)std::max<int64_t>(1, std::min<int64_t>((n + kThreads - 1) / kThreads, cap));
         // the dense core, if one pays: its rows' head records stream nothing
         TC_TRY(core_setup(g, dh, flags, s));
         const int64_t core_t = n - g->core_c;
-        if (narrow) {
+        if (g->narrow()) {
             TC_TRY(build_runs(g, s, m, n, bits, keys, slot, dh, hptr, big, nbig, (uint32_t*)hnext,
-                              (uint32_t*)tnext, rows_blocks, core_t));
+                              (uint32_t*)tnext, core_t));
         } else {
             TC_TRY(build_runs(g, s, m, n, bits, keys, slot, dh, hptr, big, nbig, (unsigned long long*)hnext,
-                              (unsigned long long*)tnext, rows_blocks, core_t));
+                              (unsigned long long*)tnext, core_t));
         }
     } else if (n > 0) {
         // no edges: every row is empty

@@ -215,14 +215,16 @@ __global__ void k_export_tri(const ull* __restrict__ tri, const int32_t* __restr
         out[perm[r]] = tri[r];
 }
 
-__global__ void k_export_flags(const uint32_t* __restrict__ flag, const int64_t* __restrict__ edge_tail,
+template <class P>
+__global__ void k_export_flags(const uint32_t* __restrict__ flag, const P* __restrict__ edge_tail,
                                int64_t m, uint8_t* __restrict__ out) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
          e += (int64_t)gridDim.x * blockDim.x)
         out[e] = flag_get(flag, edge_tail[e]) ? 1 : 0;
 }
 
-__global__ void k_export_edge_counts(const uint32_t* __restrict__ ecnt, const int64_t* __restrict__ edge_tail,
+template <class P>
+__global__ void k_export_edge_counts(const uint32_t* __restrict__ ecnt, const P* __restrict__ edge_tail,
                                      int64_t m, uint32_t* __restrict__ out) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
          e += (int64_t)gridDim.x * blockDim.x)
@@ -245,7 +247,8 @@ __global__ void k_import_tri(const uint64_t* __restrict__ in, const int32_t* __r
     if ((threadIdx.x & 31) == 0 && local) atomicAdd(sum, local);
 }
 
-__global__ void k_import_flags(const uint8_t* __restrict__ in, const int64_t* __restrict__ edge_tail, int64_t m,
+template <class P>
+__global__ void k_import_flags(const uint8_t* __restrict__ in, const P* __restrict__ edge_tail, int64_t m,
                                uint32_t* __restrict__ flag) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
          e += (int64_t)gridDim.x * blockDim.x)
@@ -258,6 +261,10 @@ inline int blocks_for(int64_t items, int threads) {
     if (b < 1) b = 1;
     return (int)(b < cap ? b : cap);
 }
+
+// One block per 256 rows, started in order: a union's rows in work at a time
+// belong to few graphs, whose counts and flags then stay in L2.
+inline int ordered_blocks(int64_t n) { return (int)std::max<int64_t>(1, (n + 255) / 256); }
 
 }  // namespace
 
@@ -278,7 +285,7 @@ tc_status run_centrality(tc_graph* g, uint64_t* d_numer, double* d_tc, cudaStrea
     const int64_t small = list ? n : g->band[0];
     if (small > 0) {
         launch_scope ls("gather_thread", s);
-        k_gather_thread<<<blocks_for(small, 256), 256, 0, s>>>(a, small);
+        k_gather_thread<<<ordered_blocks(small), 256, 0, s>>>(a, small);
         TC_LAUNCH_CHECK();
     }
     if (mids > 0) {
@@ -314,7 +321,7 @@ tc_status run_divide(const uint64_t* d_numer, int64_t n, uint64_t den, double* d
 tc_status export_tri(tc_graph* g, uint64_t* d_tri, cudaStream_t s) {
     if (g->n == 0) return TC_OK;
     launch_scope ls("export_tri", s);
-    k_export_tri<<<blocks_for(g->n, 256), 256, 0, s>>>(g->tri, g->perm, g->n, (ull*)d_tri);
+    k_export_tri<<<ordered_blocks(g->n), 256, 0, s>>>(g->tri, g->perm, g->n, (ull*)d_tri);
     TC_LAUNCH_CHECK();
     return TC_OK;
 }
@@ -323,7 +330,10 @@ tc_status export_edge_counts(tc_graph* g, uint32_t* d_out, cudaStream_t s) {
     if (g->m == 0) return TC_OK;
     if (!g->ecnt) return TC_ERR_STATE;
     launch_scope ls("export_edge_counts", s);
-    k_export_edge_counts<<<blocks_for(g->m, 256), 256, 0, s>>>(g->ecnt, g->edge_tail, g->m, d_out);
+    if (g->narrow())
+        k_export_edge_counts<<<blocks_for(g->m, 256), 256, 0, s>>>(g->ecnt, (const uint32_t*)g->edge_tail, g->m, d_out);
+    else
+        k_export_edge_counts<<<blocks_for(g->m, 256), 256, 0, s>>>(g->ecnt, (const ull*)g->edge_tail, g->m, d_out);
     TC_LAUNCH_CHECK();
     return TC_OK;
 }
@@ -339,7 +349,10 @@ tc_status import_counts(tc_graph* g, const uint64_t* d_tri, const uint8_t* d_fla
     }
     if (m > 0) {
         launch_scope ls("import_flags", s);
-        k_import_flags<<<blocks_for(m, 256), 256, 0, s>>>(d_flag, g->edge_tail, m, g->flag);
+        if (g->narrow())
+            k_import_flags<<<blocks_for(m, 256), 256, 0, s>>>(d_flag, (const uint32_t*)g->edge_tail, m, g->flag);
+        else
+            k_import_flags<<<blocks_for(m, 256), 256, 0, s>>>(d_flag, (const ull*)g->edge_tail, m, g->flag);
         TC_LAUNCH_CHECK();
     }
     return TC_OK;
@@ -348,7 +361,10 @@ tc_status import_counts(tc_graph* g, const uint64_t* d_tri, const uint8_t* d_fla
 tc_status export_flags(tc_graph* g, uint8_t* d_flag, cudaStream_t s) {
     if (g->m == 0) return TC_OK;
     launch_scope ls("export_flags", s);
-    k_export_flags<<<blocks_for(g->m, 256), 256, 0, s>>>(g->flag, g->edge_tail, g->m, d_flag);
+    if (g->narrow())
+        k_export_flags<<<blocks_for(g->m, 256), 256, 0, s>>>(g->flag, (const uint32_t*)g->edge_tail, g->m, d_flag);
+    else
+        k_export_flags<<<blocks_for(g->m, 256), 256, 0, s>>>(g->flag, (const ull*)g->edge_tail, g->m, d_flag);
     TC_LAUNCH_CHECK();
     return TC_OK;
 }

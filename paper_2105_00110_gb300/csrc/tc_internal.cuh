@@ -15,7 +15,8 @@
 //                         the part of N_H(u) that can close a triangle with
 //                         the oriented edge u -> v.  col[] is not written at
 //                         head positions; tail positions hold N_H(v) ascending
-//   edge_tail[m]  int64   canonical edge e -> its tail position in rank space
+//   edge_tail[m]  uint32  canonical edge e -> its tail position in rank space
+//                         (uint64 from m = 2^31 on)
 //   flag[2m/32]   uint32  one bit per CSR position: the in-a-triangle flag of
 //                         each edge, on its tail entry (65 MB at m = 2.6e8,
 //                         small enough to stay in L2 while the count runs)
@@ -106,7 +107,8 @@ struct tc_graph {
     int32_t* col = nullptr;
     int64_t* hstart = nullptr;
     tc_head* head = nullptr;
-    int64_t* edge_tail = nullptr;
+    void* edge_tail = nullptr;           // uint32_t while 2m < 2^32 (narrow), else uint64_t
+    bool narrow() const { return 2 * m < ((int64_t)1 << 32); }
     int64_t* work = nullptr;             // [n] W(v) = Σ_{u ∈ N_L(v)} hrem(u, v)
     // rows by degree: up to 32, up to 4096 (mid), above (hub).  A single graph's
     // degrees ascend with rank: band holds the first mid and the first hub
@@ -327,7 +329,6 @@ typedef std::function<tc_status(void**, size_t)> sort_alloc;
 int sort_first_digit(int64_t np, int bits);
 tc_status sort_keys_msd(const sort_alloc& get, uint64_t* keys, uint64_t* other, uint32_t* first_counts, int64_t np,
                         int bits, const unsigned int* err, uint64_t** sorted, int64_t* valid, cudaStream_t s);
-
 // dense core (tc_core.cu).  Build flag for unions of many graphs, which
 // have no dense core: the build never sets one up.
 constexpr uint32_t TC_BUILD_NO_CORE = 1u << 30;
