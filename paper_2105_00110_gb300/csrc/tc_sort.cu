@@ -20,7 +20,6 @@
 // buffer at its place, so the buffer is the sorted array.  Keys of all ones
 // (self-loops) are dropped by the first scatter.
 #include <algorithm>
-#include <mutex>
 #include <utility>
 
 #include "tc_internal.cuh"
@@ -526,20 +525,11 @@ int sort_first_digit(int64_t np, int bits) {
 
 tc_status sort_keys_msd(const sort_alloc& get, uint64_t* keys, uint64_t* other, uint32_t* first_counts, int64_t np,
                         int bits, const unsigned int* err, uint64_t** sorted, int64_t* valid, cudaStream_t s) {
-    // the kernels' shared-memory limits, raised once
-    static std::once_flag once;
-    static cudaError_t attr = cudaSuccess;
-    std::call_once(once, [] {
-        const std::pair<const void*, size_t> fn[] = {{(const void*)k_scatter<true>, part_smem()},
-                                                     {(const void*)k_scatter<false>, part_smem()},
-                                                     {(const void*)k_sort_local<512, kLocalCap>, local_smem(kLocalCap)}};
-        for (const auto& f : fn) {
-            const cudaError_t e =
-                cudaFuncSetAttribute(f.first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.second);
-            if (e != cudaSuccess) attr = e;
-        }
-    });
-    TC_CUDA(attr);
+    // shared-memory limits (of the current device, so set on each call)
+    TC_CUDA(cudaFuncSetAttribute(k_scatter<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)part_smem()));
+    TC_CUDA(cudaFuncSetAttribute(k_scatter<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)part_smem()));
+    TC_CUDA(cudaFuncSetAttribute(k_sort_local<512, kLocalCap>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)local_smem(kLocalCap)));
     const int want = digits_wanted(np), d0 = sort_first_digit(np, bits), sms = sm_count();
     int64_t *one = nullptr, *total = nullptr;
     unsigned int* num = nullptr;
