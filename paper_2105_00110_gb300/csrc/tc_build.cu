@@ -328,7 +328,7 @@ __device__ __forceinline__ void write_tail(int64_t r, int64_t t, int64_t e, uint
     // core's product counts those triangles
     rec.hrem = r >= core_t ? 0 : (int32_t)(e - t - 1);
     rec.twin = t;
-    head[hp] = rec;   // one 16-byte store
+    store_head(head + hp, rec);
 }
 
 template <class C>

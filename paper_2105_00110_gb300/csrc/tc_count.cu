@@ -265,7 +265,7 @@ __device__ __forceinline__ entry fetch_entry(int64_t p, int64_t pe, const tc_hea
                                              const tc_dims& dm) {
     entry e{0, 0, 0};
     if (p < pe) {
-        const tc_head rec = head[TC_IX(p, dm.e2)];   // one 16-byte load
+        const tc_head rec = load_head(head + TC_IX(p, dm.e2));
         e.r = rec.hrem;
         e.t = rec.twin;
         e.u = rec.u;
@@ -684,7 +684,7 @@ k_count_warp(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ co
         const int64_t lim = min(base + fetch, n_items);
         for (int64_t it = base; it < lim; ++it) {
             const int64_t gi = it_off + it_stride * it;   // this shard's it-th item
-            const tc_item d = it_d[gi];
+            const tc_item d = load_item(it_d + gi);
             const int32_t v = d.v, nbits = it_nb[gi];
             const int64_t pb = it_pb[gi], pe = it_pe[gi];
             entry nxt = fetch_entry(pb + lane, pe, head, dm);
@@ -785,7 +785,7 @@ k_count_cta(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col
         const int64_t it = s_item;
         if (it >= n_items) break;
         const int64_t gi = it_off + it_stride * it;   // this shard's it-th item
-        const tc_item d = it_d[gi];
+        const tc_item d = load_item(it_d + gi);
         const int32_t v = d.v;
         const int64_t pb = it_pb[gi], pe = it_pe[gi];
         entry nxt = fetch_entry(pb + t, pe, head, dm);
@@ -924,7 +924,7 @@ k_count_thread(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ 
     ull tv_all = 0;
     for (int64_t it = blockIdx.x * (int64_t)blockDim.x + t; it < n_items; it += (int64_t)gridDim.x * blockDim.x) {
         const int64_t gi = it_off + it_stride * it;   // this shard's it-th item
-        const tc_item d = it_d[gi];
+        const tc_item d = load_item(it_d + gi);
         if (d.hv < MINH || d.hv > MAXH) continue;   // another launch's item
         const int32_t v = d.v;
         const int64_t h0 = d.h0;
@@ -952,10 +952,10 @@ k_count_thread(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ 
                 first[j] = j < r.hrem ? col[TC_IX(r.twin + 1 + j, dm.e2)] : 0;
         };
         if (pb < pe) {
-            nrec = head[TC_IX(pb, dm.e2)];
+            nrec = load_head(head + TC_IX(pb, dm.e2));
             fetch_first(nrec);
             rec = nrec;
-            if (pb + 1 < pe) nrec = head[TC_IX(pb + 1, dm.e2)];
+            if (pb + 1 < pe) nrec = load_head(head + TC_IX(pb + 1, dm.e2));
         }
         for (int64_t p = pb; p < pe; ++p) {
             const int64_t q0 = rec.twin + 1;
@@ -967,7 +967,7 @@ k_count_thread(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ 
             if (p + 1 < pe) {
                 rec = nrec;
                 fetch_first(rec);
-                if (p + 2 < pe) nrec = head[TC_IX(p + 2, dm.e2)];
+                if (p + 2 < pe) nrec = load_head(head + TC_IX(p + 2, dm.e2));
             }
             uint32_t hits = 0;
             // first staged id not below the stream's first id (bisection)
@@ -1268,7 +1268,7 @@ k_emit(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hstart, 
                 const tc_item d{h0, (int32_t)r, (int32_t)(h1 - h0)};
                 const int32_t nbits = h1 > h0 ? col[h1 - 1] - (int32_t)r : 0;
                 for (int64_t j = 0; j < k; ++j) {
-                    tg.d[c][at + j] = d;
+                    store_item(tg.d[c] + at + j, d);
                     tg.nb[c][at + j] = nbits;
                     tg.pb[c][at + j] = b + lv * j / k;
                     tg.pe[c][at + j] = b + lv * (j + 1) / k;

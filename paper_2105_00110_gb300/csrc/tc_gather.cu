@@ -103,7 +103,7 @@ __device__ __forceinline__ ull tri_of(const gather_args& a, int32_t u) {
 // gives u and the twin position holding its flag, a tail entry holds u in
 // col and its flag in place.
 __device__ __forceinline__ ull head_term(const gather_args& a, int64_t p) {
-    const tc_head rec = a.head[TC_IX(p, a.dm.e2)];
+    const tc_head rec = load_head(a.head + TC_IX(p, a.dm.e2));
     return (flag_get(a.flag, TC_IX(rec.twin, a.dm.fw * 32)) ? 1ull : 3ull) * tri_of(a, rec.u);
 }
 __device__ __forceinline__ ull tail_term(const gather_args& a, int64_t p) {

@@ -75,11 +75,31 @@ struct tc_plan_params {
 // What a count kernel needs of an item's middle vertex v, in one 16-byte
 // load: where N_H(v) starts in the CSR and how long it is (so that staging
 // does not wait on two dependent loads of row_ptr and hstart first).
-struct tc_item {
+struct __align__(16) tc_item {
     int64_t h0;    // hstart[v]
     int32_t v;
     int32_t hv;    // |N_H(v)|
 };
+
+#ifdef __CUDACC__
+// Records of 16 bytes move as one vector each.  (Copied as structs they went as
+// two 8-byte accesses; the stores of head records, one a tail at random
+// places, then cost two sectors each.)
+__device__ __forceinline__ void store_head(tc_head* p, tc_head x) {
+    *reinterpret_cast<int4*>(p) = make_int4(x.u, x.hrem, (int)x.twin, (int)(x.twin >> 32));
+}
+__device__ __forceinline__ tc_head load_head(const tc_head* p) {
+    const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+    return tc_head{v.x, v.y, (int64_t)(((uint64_t)(uint32_t)v.w << 32) | (uint32_t)v.z)};
+}
+__device__ __forceinline__ void store_item(tc_item* p, tc_item x) {
+    *reinterpret_cast<int4*>(p) = make_int4((int)x.h0, (int)(x.h0 >> 32), x.v, x.hv);
+}
+__device__ __forceinline__ tc_item load_item(const tc_item* p) {
+    const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+    return tc_item{(int64_t)(((uint64_t)(uint32_t)v.y << 32) | (uint32_t)v.x), v.z, v.w};
+}
+#endif
 
 struct tc_plan {
     int strategy = -1;                 // strategy the plan was made for
