@@ -394,6 +394,10 @@ constexpr int kMidShort = TC_MID_SHORT;   // longest run of the one-warp tier (5
 // at most n runs; more than kMidRun tails after those n entries for
 // k_runs_big (count nbig[2], fewer than m / kMidRun).
 constexpr int kSmallTails = 512;   // tails a warp holds at a time
+// A warp takes 32 rows from this many rows an SM on, where they fill the
+// device's warps, and four below, in CTAs of one warp: the 4096 rows of R-MAT
+// scale 12 were 128 warps on 16 SMs (36 -> 12 us; scale 16, 431 rows an SM, 44 -> 38).
+constexpr int64_t kSmallRowsFrom = 1024;
 struct small_runs {
     int64_t p0[32];      // first tail of each row's run in slot
     int64_t hs[32];      // row split: first tail position
@@ -408,16 +412,16 @@ k_runs_small(const int64_t* __restrict__ row_ptr, const int64_t* __restrict__ hs
              const int64_t* __restrict__ hptr, const uint64_t* __restrict__ slot, int64_t n,
              C* __restrict__ hnext, int32_t* __restrict__ col, tc_head* __restrict__ head,
              C* __restrict__ edge_tail, int32_t* __restrict__ big,
-             unsigned int* __restrict__ nbig, int64_t core_t) {
+             unsigned int* __restrict__ nbig, int64_t core_t, int rows) {
     __shared__ small_runs s_runs[kThreads / 32];
     small_runs& sr = s_runs[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t base = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 32; base < n;
-         base += warps * 32) {
+    for (int64_t base = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * rows; base < n;
+         base += warps * rows) {
         const int64_t r = base + lane;
         int len = 0;
-        if (r < n) {
+        if (lane < rows && r < n) {
             const int64_t p0 = hptr[r], L = hptr[r + 1] - p0;
             if (L > kMidRun) big[n + (int64_t)atomicAdd(&nbig[2], 1u)] = (int32_t)r;
             else if (L > kMidShort) big[n - 1 - (int64_t)atomicAdd(&nbig[1], 1u)] = (int32_t)r;
@@ -981,8 +985,10 @@ tc_status build_runs(tc_graph* g, cudaStream_t s, int64_t m, int64_t n, int bits
     }
     {
         launch_scope ls("build_runs_small", s);
-        k_runs_small<<<ordered_blocks(n, kThreads), kThreads, 0, s>>>(g->row_ptr, g->hstart, hptr, slot, n, hnext, g->col,
-                                                      g->head, (C*)g->edge_tail, big, nbig, core_t);
+        const int rows = n < (int64_t)sm_count() * kSmallRowsFrom ? 4 : 32;
+        const int64_t warps = (n + rows - 1) / rows, per = rows == 32 ? kThreads / 32 : 1;
+        k_runs_small<<<ordered_blocks(warps, per), (int)(32 * per), 0, s>>>(
+            g->row_ptr, g->hstart, hptr, slot, n, hnext, g->col, g->head, (C*)g->edge_tail, big, nbig, core_t, rows);
         TC_LAUNCH_CHECK();
     }
     {
