@@ -398,6 +398,7 @@ tc_status tc_set_plan_params(tc_graph* g, const int64_t* params3) {
     g->params.cta_min_work = params3[0];
     g->params.cta_chunk = params3[1];
     g->params.warp_chunk = params3[2];
+    g->params.warp_split = INT64_MAX;   // the caller's target holds
     g->params_version += 1;   // the next count re-plans
     return TC_OK;
 }

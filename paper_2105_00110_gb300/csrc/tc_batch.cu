@@ -256,7 +256,8 @@ tc_status tc_batch_autotune(tc_batch* b, int reps, tc_stream stream) {
     tc_status st = TC_OK;
     for (const tc_plan_params& c : cands) {
         g->params = c;
-        g->params.thread_work = best_p.thread_work;   // not one of the tuned settings
+        g->params.thread_work = best_p.thread_work;   // not tuned settings
+        g->params.warp_split = best_p.warp_split;
         g->params_version += 1;
         st = run_count(g, s);   // re-plans for the new parameters, then warms up
         if (st < 0) break;

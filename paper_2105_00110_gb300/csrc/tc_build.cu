@@ -1338,6 +1338,12 @@ tc_status build_graph(tc_graph* g, const void* src, const void* dst, int64_t np,
     {
         const double per = S.wedges / (64.0 * (double)sm_count());
         g->params.cta_chunk = (int64_t)std::min(4194304.0, std::max(65536.0, per));
+        // Of few wedges, the longest warp items, of up to 4096, set the count's
+        // time: smaller ones, by the same measure (a count: R-MAT scale 12 98 ->
+        // 74 us, 16 274 -> 174, 300^2 grid 203 -> 83, 600^2 grid 482 -> 145).
+        // With more every warp has several and the staging counts: R-MAT
+        // scale 17, at 9000 a warp's share, 256 us, 272 in items of 512.
+        if (per < 4096.0) g->params.warp_split = (int64_t)std::min(512.0, std::max(128.0, per));
     }
     // Unions of many small graphs hold millions of light vertices; one
     // thread each for those of up to 128 ids of work instead of 64 (the

@@ -1062,7 +1062,7 @@ __device__ __forceinline__ int classify_row(int64_t b, int64_t h, int64_t e, int
 // Items a vertex of class c is split into: its work over the class's chunk,
 // at most one per lower neighbour.
 __device__ __forceinline__ int64_t chunks_of(int c, int64_t lv, int64_t W, const tc_plan_params& pp) {
-    const int64_t chunk = c == TC_CLS_WARP ? pp.warp_chunk : pp.cta_chunk;
+    const int64_t chunk = c != TC_CLS_WARP ? pp.cta_chunk : pp.warp_chunk < pp.warp_split ? pp.warp_chunk : pp.warp_split;
     int64_t k = c == TC_CLS_THREAD ? 1 : (W + chunk - 1) / chunk;
     if (k > lv) k = lv;
     return k < 1 ? 1 : k;

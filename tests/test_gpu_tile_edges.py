@@ -164,3 +164,28 @@ def test_sort_rejects_a_bad_id():
         with pytest.raises(tcg.TCError) as e:
             tcg.Graph(torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), 1000)
         assert e.value.status == tcg.TC_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("scale,short", [(14, 1), (14, 0), (17, 0)])
+def test_small_graph_rules(scale, short):
+    # below 1024 vertices an SM a warp takes 4 rows of short runs instead of
+    # 32; below 4096 wedges a warp's share warp items are split beyond the
+    # target in the plan parameters, which holds once a caller sets it
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    s, d, n = gg.rmat(scale, seed=9)
+    n = max(n, 1024 * sms - short)
+    ref = oracle.run(s, d, n)
+    g = tcg.Graph(torch.from_numpy(s).cuda(), torch.from_numpy(d).cuda(), n)
+    try:
+        st = g.stats()
+        tri, flags, total, _ = g.count()
+        numer, tc, _, _ = g.centrality()
+        assert np.array_equal(tri.cpu().numpy(), ref["tri"]) and total == ref["total"]
+        assert np.array_equal(numer.cpu().numpy(), ref["numer"])
+        assert np.array_equal(tc.cpu().numpy(), ref["tc"], equal_nan=True)
+        tcg.tc_set_plan_params(g.h, **tcg.tc_get_plan_params(g.h))
+        again, _, _, _ = g.count()
+        assert np.array_equal(again.cpu().numpy(), ref["tri"])
+        assert (g.stats()["items"][2] < st["items"][2]) == (st["wedges"] / (64.0 * sms) < 4096.0)
+    finally:
+        g.close()
