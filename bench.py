@@ -405,17 +405,19 @@ def run_ours(args, spec, wl_name):
         # the build (rows a1-a2) against two byte models: what it must read
         # and write at least once (pairs in; col, head records, edge_tail,
         # the canonical edge list, row_ptr/hstart/perm/work out), and what
-        # this implementation moves (the radix passes over 8-byte keys, the
+        # this implementation moves (the sort passes over 8-byte keys, the
         # placement and run sorts, the scatter of 16- and 8-byte records at
         # 32-byte sector granularity)
         build_ms = sum(v for k, v in kernel_ms.items() if k.startswith(("build", "plan")))
         bits = max(1, int(n - 1).bit_length())
-        passes = (2 * bits + 7) // 8
+        # from 2^19 pairs on: two partition passes, one of them with a
+        # histogram read, and the local sort; below it the library's radix passes
+        passes = (2 * bits + 7) // 8 if np_pairs < (1 << 19) else 3.5
         b_min = 8.0 * np_pairs + 40.0 * m + 28.0 * n
         b_impl = (24.0 + 16.0 * passes) * np_pairs + 140.0 * m + 28.0 * n
         build_roof = None
         if build_ms > 0:
-            build_roof = {"t_ms": round(build_ms, 3), "radix_passes": passes,
+            build_roof = {"t_ms": round(build_ms, 3), "sort_passes": passes,
                           "compulsory_bytes": b_min, "compulsory_frac": round(b_min / (build_ms / 1e3) / 1e9 / peak, 4),
                           "implementation_bytes": b_impl,
                           "implementation_frac": round(b_impl / (build_ms / 1e3) / 1e9 / peak, 4),
