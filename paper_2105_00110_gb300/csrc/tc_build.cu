@@ -3,7 +3,8 @@
 //
 //  1. pairs -> canonical keys (min, max); self-loops become a sentinel
 //     (the set-up of section "Comparison": symmetrised, loop-free, simple)
-//  2. radix sort + unique -> the m undirected edges, caller labels
+//  2. sort (tc_sort.cu; small inputs: CUB) + unique -> the m undirected
+//     edges, caller labels
 //  3. degrees; π = sort by (degree, label) (section "Notation")
 //  4. every edge relabelled by π and placed in the run of its lower end;
 //     each run sorted (warp registers, a warp's shared region or a CTA,
@@ -14,8 +15,9 @@
 //  6. planner: per middle vertex v its work W(v) = Σ_{u∈N_L(v)} hrem, and
 //     the work items of the count step, heavy vertices split into chunks
 //
-// Radix sorts (steps 2-3) and scans use CUB (header-only, compiled into
-// this library); the per-row run sorts are this file's own.
+// The radix sorts of small inputs and of the degree order, the unique step
+// and the scans use CUB (header-only, compiled into this library); the per-row
+// run sorts are this file's own.
 #include <cub/cub.cuh>
 
 #include <algorithm>
@@ -393,11 +395,13 @@ constexpr int kMidShort = TC_MID_SHORT;   // longest run of the one-warp tier (5
 // a tail's place in its run is the number of smaller ones there (they are
 // distinct), counted by reading the run, whose lanes share those reads.  So
 // every lane works however short the runs are, and four tails' cursor atomics
-// and stores a lane are in flight together.  Bound by the latency of those
-// scattered stores and by issue; a network over the warp's registers, eight
+// and stores a lane are in flight together.  Bound by those scattered stores,
+// a sector each in L2 and DRAM (more of them in flight a lane changed nothing);
+// a network over the warp's registers, eight
 // runs at a time with a run in the first lanes of each register, kept 3 of 32
 // lanes busy on the 8192-graph batch (4096^2 grid: 6.4 -> 5.6 ms; with the
-// blocks in order 4.5, and 12.3 -> 7.1 on the batch).
+// blocks in order 4.5, and 12.3 -> 7.1 on the batch; with head records stored
+// whole 4.4 and 6.5).
 // Longer runs are queued: 33..kMidShort tails from the front of `big`
 // (count nbig[0]) and kMidShort+1..kMidRun tails from the back of its first
 // n entries (count nbig[1]) for k_runs_mid, which never meet since there are
